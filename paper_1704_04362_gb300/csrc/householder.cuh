@@ -1,0 +1,44 @@
+// Householder QR of batched slices (householder.cu).
+#pragma once
+
+#include "tp_internal.cuh"
+
+namespace tp {
+
+constexpr int HQR_MAX_L = 96;   // columns of a slice
+
+// Split planes (p0 non-null): Q also leaves as the hi/lo planes (bf16 or
+// tf32, dftc::put_split) of the next tensor-core product's B operand,
+// K-major with leading dimension ldk, p <= ldk <= 32 ceil(p / 32) (rows
+// p .. ldk-1 and the columns from l on zero), slice stride ldk * lfull --
+// the operand split fused.
+struct HqrSplit {
+  float* p0;
+  float* p1;
+  float* p2;
+  float* p3;
+  int64_t ldk;
+  int bf16;
+};
+
+// Whether householder_launch takes slices of p x l (else householder_tall_launch).
+bool householder_applies(int64_t p, int64_t l);
+
+// Orthonormalises `batch` slices Y (p x l, column-major, slice stride sY) in
+// place.  lcols (device, per slice, or null): only the first lcols[f] columns
+// are factored, the others set to zero.  keep_phase: column j of Q is
+// multiplied by sign(R(j, j)) (R's diagonal is real), so that for Y with
+// nearly orthonormal columns Q(:, j) stays close to Y(:, j) instead of
+// possibly flipping its sign.
+int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
+                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{});
+
+// The same for contiguous slices of more than 256 rows (slice stride rows * l),
+// with `scratch` of householder_tall_scratch() bytes, 256-byte aligned.  A
+// slice that is all zero or not finite sets TP_DEV_BREAKDOWN and is left zero
+// (not a number).
+size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch);
+int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
+                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st);
+
+}  // namespace tp

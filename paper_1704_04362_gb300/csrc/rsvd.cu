@@ -6,17 +6,15 @@
 //   U_f = Q W[:, :k],  V_f = V_B[:, :k],  S_f = diag(s[:k])
 // followed by the inverse DFT of U, S, V (Theorem 2.6's form, tubal rank k).
 // The test matrix has random-sign entries from Philox stream 2 (see
-// tsvd_randomized in tprod.h).  orth() is a float32 Householder QR in shared
-// memory for slices of at most 256 rows; taller slices take CholeskyQR2
-// (Fukaya et al. 2014): G = Y^H Y and its Cholesky factor R in float64,
-// Y <- Y R^{-1}, twice; if a Cholesky fails, the Gram matrix is shifted
-// (shifted CholeskyQR, Fukaya et al. 2020) and one more pass is made; a
-// failure after that sets TP_DEV_BREAKDOWN.  Every product with X_hat is a plain column-major batched
-// complex GEMM because X_hat^H is formed once.
+// tsvd_randomized in tprod.h).  orth() is a float32 Householder QR
+// (householder.cu): one CTA per slice of at most 256 rows, a tree of them for
+// taller slices.  Every product with X_hat is a plain
+// column-major batched complex GEMM because X_hat^H is formed once.
 #include <cfloat>
 #include <cmath>
 
 #include "dft_common.cuh"
+#include "householder.cuh"
 #include "philox.cuh"
 
 namespace tp {
@@ -27,8 +25,6 @@ int jacobi_double_launch(double* gr, double* gi, int64_t sG, double* vr, double*
                          const int* real_flags, int32_t* status, cudaStream_t st);
 
 namespace {
-
-constexpr int QR_THREADS = 256;
 
 // X^H of every slice: out(j, i) = conj(in(i, j)), in n1 x n2, out n2 x n1.
 __global__ void conj_transpose_kernel(const float* __restrict__ ir, const float* __restrict__ ii,
@@ -132,420 +128,6 @@ __global__ void sketch_kernel(float* __restrict__ om_r, float* __restrict__ om_i
     const bool real = f == 0 || (n3 % 2 == 0 && f == h - 1);
     om_r[e] = real ? s0 : s0 * inv_sqrt2;
     om_i[e] = real ? 0.f : s1 * inv_sqrt2;
-  }
-}
-
-// Gram of the columns of Y (p x l, float32 planar, column-major) into
-// G (l x l, float64, interleaved re/im, full Hermitian).
-__device__ void gram(const float* __restrict__ yr, const float* __restrict__ yi, int p, int l,
-                     double* G) {
-  const int npairs = l * (l + 1) / 2;
-  for (int e = threadIdx.x; e < npairs; e += blockDim.x) {
-    // e -> (a, b), a <= b, row-major upper triangle
-    int a = 0, rem = e;
-    while (rem >= l - a) { rem -= l - a; ++a; }
-    const int b = a + rem;
-    const float* xa_r = yr + int64_t(a) * p;
-    const float* xa_i = yi + int64_t(a) * p;
-    const float* xb_r = yr + int64_t(b) * p;
-    const float* xb_i = yi + int64_t(b) * p;
-    double sr = 0.0, si = 0.0;
-    for (int r = 0; r < p; ++r) {
-      const double ar = xa_r[r], ai = xa_i[r], br = xb_r[r], bi = xb_i[r];
-      sr += ar * br + ai * bi;
-      si += ar * bi - ai * br;
-    }
-    G[2 * (a * l + b)] = sr;
-    G[2 * (a * l + b) + 1] = si;
-    G[2 * (b * l + a)] = sr;
-    G[2 * (b * l + a) + 1] = -si;
-  }
-}
-
-// In-place upper Cholesky G = R^H R (R in the upper triangle of G).
-// Returns false on a non-positive pivot.
-__device__ bool cholesky(double* G, int l, int* fail) {
-  for (int j = 0; j < l; ++j) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double d = G[2 * (j * l + j)];
-      for (int i = 0; i < j; ++i) {
-        const double rr = G[2 * (i * l + j)], ri = G[2 * (i * l + j) + 1];
-        d -= rr * rr + ri * ri;
-      }
-      if (!(d > 0.0) || !isfinite(d)) *fail = 1;
-      G[2 * (j * l + j)] = (d > 0.0 && isfinite(d)) ? sqrt(d) : 1.0;
-      G[2 * (j * l + j) + 1] = 0.0;
-    }
-    __syncthreads();
-    const double djj = G[2 * (j * l + j)];
-    for (int k = j + 1 + threadIdx.x; k < l; k += blockDim.x) {
-      double sr = G[2 * (j * l + k)], si = G[2 * (j * l + k) + 1];
-      for (int i = 0; i < j; ++i) {
-        // subtract conj(R_ij) R_ik
-        const double ar = G[2 * (i * l + j)], ai = G[2 * (i * l + j) + 1];
-        const double br = G[2 * (i * l + k)], bi = G[2 * (i * l + k) + 1];
-        sr -= ar * br + ai * bi;
-        si -= ar * bi - ai * br;
-      }
-      G[2 * (j * l + k)] = sr / djj;
-      G[2 * (j * l + k) + 1] = si / djj;
-    }
-  }
-  __syncthreads();
-  return *fail == 0;
-}
-
-// Y <- Y R^{-1}, row by row (x R = y by forward substitution), in place.
-__device__ void right_solve(float* yr, float* yi, int p, int l, const double* R) {
-  for (int r = threadIdx.x; r < p; r += blockDim.x) {
-    for (int j = 0; j < l; ++j) {
-      double sr = yr[r + int64_t(p) * j], si = yi[r + int64_t(p) * j];
-      for (int i = 0; i < j; ++i) {
-        const double xr = yr[r + int64_t(p) * i], xi = yi[r + int64_t(p) * i];
-        const double ar = R[2 * (i * l + j)], ai = R[2 * (i * l + j) + 1];
-        sr -= xr * ar - xi * ai;
-        si -= xr * ai + xi * ar;
-      }
-      const double d = R[2 * (j * l + j)];
-      yr[r + int64_t(p) * j] = float(sr / d);
-      yi[r + int64_t(p) * j] = float(si / d);
-    }
-  }
-}
-
-// CholeskyQR2 (with a shifted retry) of every slice's p x l block.
-__global__ void __launch_bounds__(QR_THREADS) cholqr2_kernel(float* y_re, float* y_im, int64_t sY,
-                                                             int p, int lfull,
-                                                             const int32_t* lcols,
-                                                             int32_t* status) {
-  extern __shared__ double G[];   // 2 * l * l
-  __shared__ int fail;
-  // per-slice column count (the per-frequency sketch size): the columns from
-  // l on are set to zero
-  const int l = lcols ? min(max(int(lcols[blockIdx.x]), 1), lfull) : lfull;
-  float* yr = y_re + int64_t(blockIdx.x) * sY;
-  float* yi = y_im + int64_t(blockIdx.x) * sY;
-  for (int64_t e = int64_t(p) * l + threadIdx.x; e < int64_t(p) * lfull; e += blockDim.x) {
-    yr[e] = 0.f;
-    yi[e] = 0.f;
-  }
-  int passes_left = 2;
-  bool shifted = false;
-  for (int it = 0; it < 4 && passes_left > 0; ++it) {
-    if (threadIdx.x == 0) fail = 0;
-    gram(yr, yi, p, l, G);
-    __syncthreads();
-    if (shifted) {
-      // shift s = 11 (p l + l (l + 1)) u ||Y||_F^2 on the diagonal
-      if (threadIdx.x == 0) {
-        double tr = 0.0;
-        for (int j = 0; j < l; ++j) tr += G[2 * (j * l + j)];
-        const double s = 11.0 * (double(p) * l + double(l) * (l + 1)) * 1.1102230246251565e-16 * tr;
-        for (int j = 0; j < l; ++j) G[2 * (j * l + j)] += s;
-      }
-      __syncthreads();
-    }
-    const bool ok = cholesky(G, l, &fail);
-    if (!ok) {
-      if (shifted) {
-        if (threadIdx.x == 0 && status) atomicOr(status, TP_DEV_BREAKDOWN);
-        return;
-      }
-      shifted = true;   // retry this pass with a shift, then two plain passes
-      passes_left = 3;
-      continue;
-    }
-    __syncthreads();
-    right_solve(yr, yi, p, l, G);
-    __syncthreads();
-    shifted = false;
-    --passes_left;
-  }
-}
-
-// ---------------------------------------------------------------- Householder QR in shared memory
-// orth() of one slice's Y (p x l, p >= l, float32) held in shared memory:
-// the Householder QR Y = Q R with reflectors H_j = I - tau_j v_j v_j^H
-// (v_j(j) = 1, zero above) chosen as LAPACK's zlarfg chooses them, so that
-// H_j^H maps rows j.. of column j onto beta_j e_j with beta_j real; then
-// Q = H_0 H_1 ... H_{l-1} [I_l; 0] formed in place by backward accumulation.
-// Householder QR is backward stable whatever the conditioning of Y: Q is
-// orthonormal to float32 rounding in one pass and cannot break down, and it
-// spans the columns of Y (completed by the reflectors where Y is rank
-// deficient), which is all the range finder uses.  A step's reflector sits
-// in registers (lane r % 32 holds rows r); each warp applies it to its
-// columns k = j + 1 + warp (mod warps), and the owner of column j + 1 forms
-// the next reflector at once (look-ahead), so a step costs one barrier.
-constexpr int HQR_THREADS = 256;
-constexpr int HQR_WARPS = HQR_THREADS / 32;
-constexpr int HQR_MAX_L = 96;
-
-__device__ __forceinline__ float hqr_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Two (four) warp sums at once by exchanging halves of the values at the
-// first (two) levels instead of reducing each value separately: 5 + 2
-// broadcasts (6 + 4) shuffles instead of 10 (20); every lane gets every sum.
-__device__ __forceinline__ void hqr_sum2(float& a, float& b, int lane) {
-  const bool up = lane & 16;
-  float k = up ? b : a;
-  k += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);   // a in the low half, b in the high
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  a = __shfl_sync(0xffffffffu, k, 0);
-  b = __shfl_sync(0xffffffffu, k, 16);
-}
-__device__ __forceinline__ void hqr_sum4(float (&d)[4], int lane) {
-  const bool up = lane & 16, mid = lane & 8;
-  float k0 = up ? d[2] : d[0], k1 = up ? d[3] : d[1];
-  k0 += __shfl_xor_sync(0xffffffffu, up ? d[0] : d[2], 16);
-  k1 += __shfl_xor_sync(0xffffffffu, up ? d[1] : d[3], 16);
-  float k = mid ? k1 : k0;
-  k += __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  // lanes 0-7 hold sum 0, 8-15 sum 1, 16-23 sum 2, 24-31 sum 3
-#pragma unroll
-  for (int u = 0; u < 4; ++u) d[u] = __shfl_sync(0xffffffffu, k, 8 * u);
-}
-
-// Reflector of column a (rows j .. p-1), one warp: rows j+1.. become v,
-// row j becomes beta; returns tau (0 when the column is already beta e_j with
-// beta real).
-__device__ float2 hqr_reflector(float2* a, int j, int p, int lane) {
-  const float2 al = a[j];
-  float s = 0.f;
-  for (int r = j + 1 + lane; r < p; r += 32) {
-    const float2 x = a[r];
-    s = fmaf(x.x, x.x, fmaf(x.y, x.y, s));
-  }
-  s = hqr_sum(s);
-  if (s == 0.f && al.y == 0.f) return make_float2(0.f, 0.f);
-  const float nrm = sqrtf(fmaf(al.x, al.x, fmaf(al.y, al.y, s)));
-  const float beta = al.x >= 0.f ? -nrm : nrm;
-  // v = x / (alpha - beta); |alpha - beta| >= nrm > 0 by the sign of beta
-  const float dr = al.x - beta, di = al.y;
-  const float den = fmaf(dr, dr, di * di);
-  const float sr = dr / den, si = -di / den;
-  for (int r = j + 1 + lane; r < p; r += 32) {
-    const float2 x = a[r];
-    a[r] = make_float2(x.x * sr - x.y * si, x.x * si + x.y * sr);
-  }
-  __syncwarp();
-  if (lane == 0) a[j] = make_float2(beta, 0.f);
-  return make_float2((beta - al.x) / beta, -al.y / beta);
-}
-
-// v_j of column a into registers: row r = lane + 32 t, 1 at row j, 0 above.
-// FULL: p == 32 RPL, so that every lane's rows exist; rows above j then
-// need no predicate (v is zero there, so they are read and rewritten
-// unchanged).
-template <int RPL, bool FULL>
-__device__ __forceinline__ void hqr_load_v(const float2* a, int j, int p, int lane,
-                                           float2 (&v)[RPL]) {
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int r = lane + 32 * t;
-    if (FULL) {
-      const float2 x = a[r];
-      v[t] = r > j ? x : make_float2(r == j ? 1.f : 0.f, 0.f);
-    } else {
-      v[t] = (r <= j || r >= p) ? make_float2(r == j ? 1.f : 0.f, 0.f) : a[r];
-    }
-  }
-}
-
-// c <- c - f v (v^H c) on rows j .. p-1 (f = conj(tau) applies H^H, f = tau H)
-template <int RPL, bool FULL>
-__device__ __forceinline__ void hqr_apply(const float2 (&v)[RPL], float2* c, int j, int p,
-                                          float2 f, int lane) {
-  float2 x[RPL];
-  float dr = 0.f, di = 0.f;
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int r = lane + 32 * t;
-    x[t] = (FULL || (r >= j && r < p)) ? c[r] : make_float2(0.f, 0.f);
-    dr = fmaf(v[t].x, x[t].x, fmaf(v[t].y, x[t].y, dr));    // Re(conj(v) x)
-    di = fmaf(v[t].x, x[t].y, fmaf(-v[t].y, x[t].x, di));   // Im(conj(v) x)
-  }
-  hqr_sum2(dr, di, lane);
-  const float gr = f.x * dr - f.y * di, gi = f.x * di + f.y * dr;
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int r = lane + 32 * t;
-    if (FULL || (r >= j && r < p))
-      c[r] = make_float2(x[t].x - (v[t].x * gr - v[t].y * gi),
-                         x[t].y - (v[t].x * gi + v[t].y * gr));
-  }
-}
-
-// hqr_apply on two columns at once (their sums interleave in the shuffles)
-template <int RPL, bool FULL>
-__device__ __forceinline__ void hqr_apply2(const float2 (&v)[RPL], float2* c0, float2* c1, int j,
-                                           int p, float2 f, int lane) {
-  float2 x0[RPL], x1[RPL];
-  float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int r = lane + 32 * t;
-    const bool in = FULL || (r >= j && r < p);
-    x0[t] = in ? c0[r] : make_float2(0.f, 0.f);
-    x1[t] = in ? c1[r] : make_float2(0.f, 0.f);
-    d[0] = fmaf(v[t].x, x0[t].x, fmaf(v[t].y, x0[t].y, d[0]));
-    d[1] = fmaf(v[t].x, x0[t].y, fmaf(-v[t].y, x0[t].x, d[1]));
-    d[2] = fmaf(v[t].x, x1[t].x, fmaf(v[t].y, x1[t].y, d[2]));
-    d[3] = fmaf(v[t].x, x1[t].y, fmaf(-v[t].y, x1[t].x, d[3]));
-  }
-  hqr_sum4(d, lane);
-  const float g0r = f.x * d[0] - f.y * d[1], g0i = f.x * d[1] + f.y * d[0];
-  const float g1r = f.x * d[2] - f.y * d[3], g1i = f.x * d[3] + f.y * d[2];
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int r = lane + 32 * t;
-    if (FULL || (r >= j && r < p)) {
-      c0[r] = make_float2(x0[t].x - (v[t].x * g0r - v[t].y * g0i),
-                          x0[t].y - (v[t].x * g0i + v[t].y * g0r));
-      c1[r] = make_float2(x1[t].x - (v[t].x * g1r - v[t].y * g1i),
-                          x1[t].y - (v[t].x * g1i + v[t].y * g1r));
-    }
-  }
-}
-
-// Column k of Q from its reflector (stored in place): H_k e_k restricted to
-// rows k.. -- 1 - tau at row k, -tau v below -- and zeros above.
-__device__ __forceinline__ void hqr_materialize(float2* a, int k, int p, float2 tau, int lane) {
-  for (int r = lane; r < p; r += 32) {
-    float2 y;
-    if (r < k) {
-      y = make_float2(0.f, 0.f);
-    } else if (r == k) {
-      y = make_float2(1.f - tau.x, -tau.y);
-    } else {
-      const float2 v = a[r];
-      y = make_float2(-(tau.x * v.x - tau.y * v.y), -(tau.x * v.y + tau.y * v.x));
-    }
-    a[r] = y;
-  }
-}
-
-// One CTA per slice; RPL rows per lane (p <= 32 RPL).
-// keep_phase: column j of Q is multiplied by sign(R(j, j)) (R's diagonal is
-// real), so that for Y with nearly orthonormal columns Q(:, j) stays close
-// to Y(:, j) instead of possibly flipping its sign.
-// Split planes (sp non-null): Q also leaves as the hi/lo planes (bf16 or
-// tf32, dftc::put_split) of the next tensor-core product's B operand,
-// K-major with leading dimension ldk >= p (rows p .. ldk-1 and the columns
-// from l on zero), slice stride ldk * lfull -- the operand split fused.
-struct HqrSplit {
-  float* p0;
-  float* p1;
-  float* p2;
-  float* p3;
-  int64_t ldk;
-  int bf16;
-};
-
-template <int RPL, bool FULL>
-__global__ void __launch_bounds__(HQR_THREADS) householder_qr_kernel(float* y_re, float* y_im,
-                                                                     int64_t sY, int p, int lfull,
-                                                                     const int32_t* lcols,
-                                                                     int keep_phase, HqrSplit sp) {
-  extern __shared__ float2 hqr_a[];   // Y, then Q: p x l column-major
-  __shared__ float2 tau_s[HQR_MAX_L];
-  __shared__ float sgn_s[HQR_MAX_L];   // sign of R(j, j)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // per-slice column count (the per-frequency sketch size): the columns from
-  // l on are left zero
-  const int l = lcols ? min(max(int(lcols[blockIdx.x]), 1), lfull) : lfull;
-  float* yr = y_re + int64_t(blockIdx.x) * sY;
-  float* yi = y_im + int64_t(blockIdx.x) * sY;
-  float2* A = hqr_a;
-  for (int e = threadIdx.x; e < p * l; e += HQR_THREADS) A[e] = make_float2(yr[e], yi[e]);
-  __syncthreads();
-  if (warp == 0) {
-    const float2 t = hqr_reflector(A, 0, p, lane);
-    if (lane == 0) {
-      tau_s[0] = t;
-      sgn_s[0] = A[0].x < 0.f ? -1.f : 1.f;
-    }
-  }
-  __syncthreads();
-  // factorisation: step j applies H_j^H to columns j+1 .. l-1
-  for (int j = 0; j + 1 < l; ++j) {
-    const float2 tau = tau_s[j];
-    float2 v[RPL];
-    hqr_load_v<RPL, FULL>(A + int64_t(j) * p, j, p, lane, v);
-    const bool live = tau.x != 0.f || tau.y != 0.f;
-    const float2 f = make_float2(tau.x, -tau.y);
-    int k = j + 1 + warp;
-    if (warp == 0) {   // look-ahead: column j + 1 first, then its reflector
-      float2* c = A + int64_t(k) * p;
-      if (live) hqr_apply<RPL, FULL>(v, c, j, p, f, lane);
-      __syncwarp();
-      const float2 t = hqr_reflector(c, k, p, lane);
-      if (lane == 0) {
-        tau_s[k] = t;
-        sgn_s[k] = c[k].x < 0.f ? -1.f : 1.f;
-      }
-      k += HQR_WARPS;
-    }
-    if (live) {
-      for (; k + HQR_WARPS < l; k += 2 * HQR_WARPS)
-        hqr_apply2<RPL, FULL>(v, A + int64_t(k) * p, A + int64_t(k + HQR_WARPS) * p, j, p, f, lane);
-      if (k < l) hqr_apply<RPL, FULL>(v, A + int64_t(k) * p, j, p, f, lane);
-    }
-    __syncthreads();
-  }
-  // Q = H_0 ... H_{l-1} [I; 0]: step i applies H_i to columns i+1 .. l-1,
-  // whose first (column i + 1) its owner first turns from reflector storage
-  // into H_{i+1} e_{i+1}
-  for (int i = l - 2; i >= 0; --i) {
-    const float2 tau = tau_s[i];
-    float2 v[RPL];
-    hqr_load_v<RPL, FULL>(A + int64_t(i) * p, i, p, lane, v);
-    int k = i + 1 + warp;
-    if (warp == 0) {
-      hqr_materialize(A + int64_t(k) * p, k, p, tau_s[k], lane);
-      __syncwarp();
-    }
-    if (tau.x != 0.f || tau.y != 0.f) {
-      for (; k + HQR_WARPS < l; k += 2 * HQR_WARPS)
-        hqr_apply2<RPL, FULL>(v, A + int64_t(k) * p, A + int64_t(k + HQR_WARPS) * p, i, p, tau, lane);
-      if (k < l) hqr_apply<RPL, FULL>(v, A + int64_t(k) * p, i, p, tau, lane);
-    }
-    __syncthreads();
-  }
-  if (warp == 0) hqr_materialize(A, 0, p, tau_s[0], lane);
-  __syncthreads();
-  for (int e = threadIdx.x; e < p * l; e += HQR_THREADS) {
-    const float2 q = A[e];
-    const float sg = keep_phase ? sgn_s[e / p] : 1.f;
-    yr[e] = sg * q.x;
-    yi[e] = sg * q.y;
-  }
-  for (int e = p * l + threadIdx.x; e < p * lfull; e += HQR_THREADS) {
-    yr[e] = 0.f;
-    yi[e] = 0.f;
-  }
-  if (sp.p0) {
-    const int64_t base = int64_t(blockIdx.x) * sp.ldk * lfull;
-    for (int64_t e = threadIdx.x; e < sp.ldk * lfull; e += HQR_THREADS) {
-      const int c = int(e / sp.ldk), r = int(e - int64_t(c) * sp.ldk);
-      float2 q = make_float2(0.f, 0.f);
-      if (r < p && c < l) {
-        q = A[c * p + r];
-        if (keep_phase) {
-          q.x *= sgn_s[c];
-          q.y *= sgn_s[c];
-        }
-      }
-      dftc::put_split(sp.p0, sp.p1, sp.bf16 != 0, base + e, q.x);
-      dftc::put_split(sp.p2, sp.p3, sp.bf16 != 0, base + e, q.y);
-    }
   }
 }
 
@@ -1199,50 +781,11 @@ unsigned grid_for(int64_t n) {
   return unsigned(b);
 }
 
-// Launch of householder_qr_kernel with RPL = 2, 4 or 8 rows per lane (p
-// up to 64, 128, 256) and the predicate-free form when p fills the lanes.
-int launch_hqr(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
-               bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{}) {
-  const size_t smem = size_t(p) * l * sizeof(float2);
-  const int kp = keep_phase ? 1 : 0;
-  const unsigned grid = unsigned(batch);
-  KernelScope ks("householder_qr", st);
-#define TP_HQR(R, F)                                                                      \
-  do {                                                                                    \
-    TP_SET_SMEM((householder_qr_kernel<R, F>), smem);                                     \
-    householder_qr_kernel<R, F><<<grid, HQR_THREADS, smem, st>>>(yr, yi, sY, p, l, lcols, kp, \
-                                                                 sp);                            \
-  } while (0)
-  if (p == 64) TP_HQR(2, true);
-  else if (p < 64) TP_HQR(2, false);
-  else if (p == 128) TP_HQR(4, true);
-  else if (p < 128) TP_HQR(4, false);
-  else if (p == 256) TP_HQR(8, true);
-  else TP_HQR(8, false);
-#undef TP_HQR
-  return launch_status("householder_qr_kernel");
-}
-
 }  // namespace
 
 // K leading dimension of the split operand planes (16-byte rows for TMA).
 int64_t split_ld(int64_t k, int prec) {
   return prec == TP_BF16X3 ? (k + 7) / 8 * 8 : (k + 3) / 4 * 4;
-}
-
-// Householder orthonormalisation of `batch` slices Y (p x l, column-major,
-// slice stride sY) in place, float32 in shared memory: p <= 256 and
-// l <= 96 (else TP_EUNSUPPORTED).  keep_phase multiplies column j by
-// sign(R(j, j)), so that nearly orthonormal columns stay close to their
-// input.
-int householder_orth_launch(float* yr, float* yi, int64_t sY, int p, int l, int64_t batch,
-                            bool keep_phase, cudaStream_t st) {
-  if (p > 256 || l > HQR_MAX_L || l > p) {
-    set_error("householder_orth: needs l <= p <= 256 and l <= %d", HQR_MAX_L);
-    return TP_EUNSUPPORTED;
-  }
-  if (batch <= 0 || l <= 0) return TP_OK;
-  return launch_hqr(yr, yi, sY, p, l, nullptr, keep_phase, batch, st);
 }
 
 size_t rsvd_ws(int64_t n1, int64_t n2, int64_t n3, int64_t k, int64_t p, int prec) {
@@ -1255,22 +798,31 @@ size_t rsvd_ws(int64_t n1, int64_t n2, int64_t n3, int64_t k, int64_t p, int pre
                                 + 4 * ws_bytes(ln * n2 * h, 4)  // X_hat^H, K-major
                                 + 4 * ws_bytes(lb * l * h, 4)   // B operand (Omega, Q or Z)
                           : 0;
+  // the tree QR of tall slices works in the space of the core's arrays
+  size_t tree = 0;
+  for (int64_t rows : {n1, n2})
+    if (!householder_applies(rows, int64_t(l))) {
+      const size_t t = householder_tall_scratch(rows, int64_t(l), int64_t(h));
+      if (t > tree) tree = t;
+    }
+  const size_t core =
+      2 * ws_bytes(size_t(n2) * l * h, 8)    // P = B^H W (Jacobi G in float64 past l = 128)
+      + 2 * ws_bytes(l * l * h, 8)           // core eigenvectors (Jacobi W)
+      + ws_bytes(l * h, 8) + ws_bytes(h, 4)  // singular values, real flags
+      + ws_bytes(size_t(QL_LOG_PER_L) * l * h, sizeof(QlRot)) + ws_bytes(h, 4)   // QL logs
+      + 2 * ws_bytes(l * size_t(k) * h, 4)   // W_k
+      + 2 * ws_bytes(size_t(n1) * k * h, 4)  // U_hat
+      + 2 * ws_bytes(size_t(k) * k * h, 4)   // S_hat
+      + 2 * ws_bytes(size_t(n2) * k * h, 4)  // V_hat
+      // slice sketch: lateral norms, picks, draw scratch
+      + ws_bytes(size_t(n2), 8) + ws_bytes(norms_partial_count(n1, n2, n3, 0), 8) +
+      ws_bytes(l, 4) + ws_bytes(l, 4) + ws_bytes(1, 8) + draw_scratch_bytes(n2);
   return split + 2 * ws_bytes(size_t(n1) * n2 * h, 4)   // X_hat
          + 2 * ws_bytes(size_t(n1) * n2 * h, 4) // X_hat^H
          + 2 * ws_bytes(size_t(n2) * l * h, 4)  // Omega
          + 2 * ws_bytes(size_t(n1) * l * h, 4)  // Y / Q
          + 2 * ws_bytes(size_t(n2) * l * h, 4)  // Z / B^H
-         + 2 * ws_bytes(size_t(n2) * l * h, 8)  // Jacobi G (float64)
-         + 2 * ws_bytes(l * l * h, 8)           // Jacobi W (float64)
-         + ws_bytes(l * h, 8) + ws_bytes(h, 4)  // singular values, real flags
-         + ws_bytes(size_t(QL_LOG_PER_L) * l * h, sizeof(QlRot)) + ws_bytes(h, 4)   // QL logs
-         + 2 * ws_bytes(l * size_t(k) * h, 4)   // W_k
-         + 2 * ws_bytes(size_t(n1) * k * h, 4)  // U_hat
-         + 2 * ws_bytes(size_t(k) * k * h, 4)   // S_hat
-         + 2 * ws_bytes(size_t(n2) * k * h, 4)  // V_hat
-         // slice sketch: lateral norms, picks, draw scratch
-         + ws_bytes(size_t(n2), 8) + ws_bytes(norms_partial_count(n1, n2, n3, 0), 8) +
-         ws_bytes(l, 4) + ws_bytes(l, 4) + ws_bytes(1, 8) + draw_scratch_bytes(n2);
+         + (core > tree ? core : tree);
 }
 
 namespace {
@@ -1447,23 +999,18 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
     planes_ready = false;
     return gemm_tc(hermitian, N, cr, ci);
   };
-  const size_t qr_smem = size_t(2) * l * l * sizeof(double);
-  TP_SET_SMEM(cholqr2_kernel, qr_smem);
   constexpr size_t kSmemCap = 200 * 1024;
   auto orth = [&](float* yr, float* yi, int64_t rows) {
-    if (rows <= 256 && l <= HQR_MAX_L) {
+    if (householder_applies(rows, l)) {
       HqrSplit sp{};
       if (tc) sp = HqrSplit{BP[0], BP[1], BP[2], BP[3], split_ld(rows, prec), bf};
       planes_ready = tc;
-      return launch_hqr(yr, yi, rows * l, int(rows), int(l), sketch_per_freq, false, h, st, sp);
+      return householder_launch(yr, yi, rows * l, int(rows), int(l), sketch_per_freq, false, h, st,
+                                sp);
     }
     planes_ready = false;
-    {
-      KernelScope ks("cholqr2", st);
-      cholqr2_kernel<<<unsigned(h), QR_THREADS, qr_smem, st>>>(yr, yi, rows * l, int(rows),
-                                                               int(l), sketch_per_freq, status);
-    }
-    return launch_status("cholqr2_kernel");
+    // the space from Gr on is written by the core only
+    return householder_tall_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
   };
 
   if (tc) {

@@ -31,11 +31,10 @@
 // Steps 2-3 are batched float64 GEMMs spread over all SMs.
 #include <atomic>
 
+#include "householder.cuh"
 #include "jacobi_rot.cuh"
 
 namespace tp {
-int householder_orth_launch(float* yr, float* yi, int64_t sY, int p, int l, int64_t batch,
-                            bool keep_phase, cudaStream_t st);
 namespace {
 using jrot::rotation;
 
@@ -998,8 +997,8 @@ int tsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, float* U, float
     // cluster at the rounding floor (rank-deficient input); the QR keeps the
     // leading columns and completes the rest to an orthonormal set
     const int64_t rows = transpose ? n2 : n1;
-    if ((rc = householder_orth_launch(transpose ? Vr : Ur, transpose ? Vi : Ui, rows * m,
-                                      int(rows), int(m), h, true, st)))
+    if ((rc = householder_launch(transpose ? Vr : Ur, transpose ? Vi : Ui, rows * m,
+                                 int(rows), int(m), nullptr, true, h, st)))
       return rc;
   }
   if ((rc = launch_irdft(Ur, Ui, n1 * m, n1 * m, n3, U, st))) return rc;
