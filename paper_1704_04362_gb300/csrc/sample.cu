@@ -8,6 +8,8 @@
 // about 44 significant bits at float32 speed; the lanes of a column are
 // combined as float pairs, partial sums in float64, all in a fixed order,
 // making every norm deterministic run to run.
+#include <algorithm>
+
 #include "philox.cuh"
 #include "tp_internal.cuh"
 
@@ -108,34 +110,59 @@ __global__ void horizontal_partial_kernel(const float* __restrict__ X, int64_t n
   partial[g * n1 + i] = double(hi) + double(lo);
 }
 
-// out[i] = sum over the G chunk partials of row i: a block takes 32 rows,
-// its 8 warps each sum a contiguous eighth of the chunks (loads batched,
-// adds in chunk order), then warp 0 adds the eight eighths in order; the
-// same partition for a given G, so every norm is deterministic.
-__global__ void __launch_bounds__(256) horizontal_reduce_kernel(const double* __restrict__ partial,
-                                                                int64_t n1, int64_t G,
-                                                                double* __restrict__ out) {
-  __shared__ double seg_sum[8][33];
-  const int lr = threadIdx.x & 31, seg = threadIdx.x >> 5;
-  const int64_t S = (G + 7) / 8;
-  for (int64_t r0 = int64_t(blockIdx.x) * 32; r0 < n1; r0 += int64_t(gridDim.x) * 32) {
+// out[i] = sum over the G chunk partials of row i (partial[g * n1 + i]; for the
+// lateral norms row j has the n3 partials of its columns): a block takes 4 rows
+// (a sector), its 64 thread groups each sum a contiguous part of the chunks
+// (loads batched, adds in chunk order), then the parts are added in order, 8
+// and 8; the same partition for a given G, so every norm is deterministic.
+// Bound by the float64 adds (two a cycle and SM), so the rows are spread over
+// as many blocks as possible: 192 rows of 4864 partials and 1140 of 168, one
+// thread a row 0.261 ms together, 32 rows a block 0.072 -> 0.038.
+constexpr int NR_ROWS = 4, NR_SEG = 64;
+
+__global__ void __launch_bounds__(NR_ROWS * NR_SEG)
+    norms_reduce_kernel(const double* __restrict__ partial, int64_t n1, int64_t G,
+                        double* __restrict__ out) {
+  __shared__ double part[NR_SEG][NR_ROWS], eighth[8][NR_ROWS];
+  const int lr = threadIdx.x % NR_ROWS, seg = threadIdx.x / NR_ROWS;
+  const int64_t S = (G + NR_SEG - 1) / NR_SEG;
+  for (int64_t r0 = int64_t(blockIdx.x) * NR_ROWS; r0 < n1; r0 += int64_t(gridDim.x) * NR_ROWS) {
     const int64_t i = r0 + lr;
     double a = 0.0;
     if (i < n1) {
-      const int64_t g1 = (seg + 1) * S < G ? (seg + 1) * S : G;
+      const int64_t g1 = min(G, (seg + 1) * S);
 #pragma unroll 8
       for (int64_t g = seg * S; g < g1; ++g) a += partial[g * n1 + i];
     }
-    seg_sum[seg][lr] = a;
+    part[seg][lr] = a;
+    __syncthreads();
+    if (seg < 8) {
+      double t = 0.0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) t += part[8 * seg + k][lr];
+      eighth[seg][lr] = t;
+    }
     __syncthreads();
     if (seg == 0 && i < n1) {
       double t = 0.0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) t += seg_sum[k][lr];
+      for (int k = 0; k < 8; ++k) t += eighth[k][lr];
       out[i] = t;
     }
-    __syncthreads();
   }
+}
+
+// Few partials per row go to lateral_reduce_kernel's one thread a row.
+void launch_norms_reduce(const double* partial, int64_t n1, int64_t G, double* out,
+                         cudaStream_t st) {
+  KernelScope ks("norms_reduce", st);
+  if (G <= 8) {
+    const int64_t rb = std::min<int64_t>((n1 + 255) / 256, int64_t(sm_count()) * 8);
+    lateral_reduce_kernel<<<unsigned(rb), 256, 0, st>>>(partial, n1, G, out);
+    return;
+  }
+  const int64_t rb = std::min<int64_t>((n1 + NR_ROWS - 1) / NR_ROWS, int64_t(sm_count()) * 8);
+  norms_reduce_kernel<<<unsigned(rb), NR_ROWS * NR_SEG, 0, st>>>(partial, n1, G, out);
 }
 
 int64_t horizontal_chunks(int64_t n1, int64_t ncols) {
@@ -441,12 +468,7 @@ int launch_slice_norms(const float* X, int64_t n1, int64_t n2, int64_t n3, int w
     int rc = tunable ? autotune_pick("norms_lateral", key, 4, 4, 2, run, st, &c) : TP_OK;
     if (!rc) rc = run(c);
     if (rc) return rc;
-    int64_t rb = (n2 + 255) / 256;
-    if (rb > int64_t(sm_count()) * 8) rb = int64_t(sm_count()) * 8;
-    {
-      KernelScope ks("norms_reduce", st);
-      lateral_reduce_kernel<<<unsigned(rb), 256, 0, st>>>(partial, n2, n3, out);
-    }
+    launch_norms_reduce(partial, n2, n3, out, st);
   } else {
     const int64_t G = horizontal_chunks(n1, ncols);
     const int64_t chunk = (ncols + G - 1) / G;
@@ -456,12 +478,7 @@ int launch_slice_norms(const float* X, int64_t n1, int64_t n2, int64_t n3, int w
       horizontal_partial_kernel<<<dim3(unsigned(bx), unsigned(G)), 256, 0, st>>>(X, n1, ncols,
                                                                                 chunk, partial);
     }
-    int64_t rb = (n1 + 31) / 32;
-    if (rb > int64_t(sm_count()) * 8) rb = int64_t(sm_count()) * 8;
-    {
-      KernelScope ks("norms_reduce", st);
-      horizontal_reduce_kernel<<<unsigned(rb), 256, 0, st>>>(partial, n1, G, out);
-    }
+    launch_norms_reduce(partial, n1, G, out, st);
   }
   return launch_status("slice_norms");
 }
