@@ -65,12 +65,16 @@ Planes take_planes(Arena& ws, size_t elems, bool tc) {
 // kk + lk*i with lk = K padded to 16 bytes (4 floats for 3xTF32, 8 bf16 for
 // BF16x3).  B_hat_k is K-major in both (leading dimension K, padded likewise
 // for the tensor cores).  The planes are sized as floats in both splits.
+size_t split_bytes(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
+  return is_tc(prec) ? ws_bytes(cgemm_split_floats(n1, n4, half_len(n3), n2, prec), 4) : 0;
+}
+
 size_t tprod_ws(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
   const size_t h = size_t(half_len(n3));
   const bool tc = is_tc(prec);
   const int64_t lk = pad_k(n2, prec);
   return planes_bytes(size_t(tc ? lk : n2) * n1 * h, tc) + planes_bytes(size_t(lk) * n4 * h, tc) +
-         2 * ws_bytes(size_t(n1) * n4 * h, 4);
+         2 * ws_bytes(size_t(n1) * n4 * h, 4) + split_bytes(n1, n2, n4, n3, prec);
 }
 
 size_t sampled_ws(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
@@ -83,7 +87,7 @@ size_t sampled_ws(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
   return 2 * ws_bytes(size_t(n2), 8) + ws_bytes(part, 8) + ws_bytes(size_t(n2), 4) +
          ws_bytes(size_t(n2), 4) + ws_bytes(1, 8) + planes_bytes(size_t(lk) * n1 * h, tc) +
          planes_bytes(size_t(lk) * n4 * h, tc) + 2 * ws_bytes(size_t(n1) * n4 * h, 4) +
-         draw_scratch_bytes(n2);
+         draw_scratch_bytes(n2) + split_bytes(n1, n2, n4, n3, prec);
 }
 
 }  // namespace
@@ -110,7 +114,10 @@ int tprod(const float* A, const float* B, float* C, int64_t n1, int64_t n2, int6
   const bool tc = is_tc(prec);
   cudaStream_t st = as_stream(stream);
   Arena ws;
-  int rc = acquire_workspace(opts, tprod_ws(n1, n2, n4, n3, prec), &ws);
+  // without the split-K partial sums a smaller workspace does (slower)
+  const size_t need = tprod_ws(n1, n2, n4, n3, prec), split = split_bytes(n1, n2, n4, n3, prec);
+  bool lean = false;
+  int rc = acquire_workspace(opts, need, &ws, need - split, &lean);
   if (rc) return rc;
   const int64_t h = half_len(n3);
   const int64_t lk = pad_k(n2, prec);              // K leading dimension
@@ -131,6 +138,8 @@ int tprod(const float* A, const float* B, float* C, int64_t n1, int64_t n2, int6
           la, lk, n1, la * (tc ? n1 : n2), lk * n4, n1 * n4, h, n3, prec,
           Ah.re_lo, Ah.im_lo, Bh.re_lo, Bh.im_lo, n2, opts ? opts->status : nullptr,
           opts ? opts->pipeline_wait_limit : 0};
+  if (split && !lean)
+    g.split_ws = ws.take<float>(cgemm_split_floats(n1, n4, h, n2, prec));
   if ((rc = launch_cgemm(g, st))) return rc;
   return launch_irdft(Cr, Ci, n1 * n4, n1 * n4, n3, C, st);
 }
@@ -167,7 +176,9 @@ int tprod_sampled(const float* A, const float* B, float* Z, int64_t n1, int64_t 
   const bool tc = is_tc(prec);
   cudaStream_t st = as_stream(stream);
   Arena ws;
-  int rc = acquire_workspace(opts, sampled_ws(n1, n2, n4, n3, prec), &ws);
+  const size_t need = sampled_ws(n1, n2, n4, n3, prec), split = split_bytes(n1, n2, n4, n3, prec);
+  bool lean = false;
+  int rc = acquire_workspace(opts, need, &ws, need - split, &lean);
   if (rc) return rc;
   const int64_t h = half_len(n3);
   const int64_t lk = pad_k(n2, prec);              // K (picked-slice) leading dimension capacity
@@ -215,6 +226,8 @@ int tprod_sampled(const float* A, const float* B, float* Z, int64_t n1, int64_t 
           la, lk, n1, la * (tc ? n1 : n2), lk * n4, n1 * n4, h, n3, prec,
           Ch.re_lo, Ch.im_lo, Rh.re_lo, Rh.im_lo, n2, opts ? opts->status : nullptr,
           opts ? opts->pipeline_wait_limit : 0};
+  if (split && !lean)
+    g.split_ws = ws.take<float>(cgemm_split_floats(n1, n4, h, n2, prec));
   if ((rc = launch_cgemm(g, st))) return rc;
   // S7: inverse transform
   return launch_irdft(Zr, Zi, n1 * n4, n1 * n4, n3, Z, st);

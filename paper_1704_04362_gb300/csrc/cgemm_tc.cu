@@ -23,6 +23,10 @@
 //                   tcgen05.ld 32x32b, add into float32 registers, mark the
 //                   set empty; after a tile's last chunk, bounds-checked
 //                   coalesced stores
+// With fewer tiles than SMs, K is cut into parts too: a work item is a tile's
+// part, the parts' sums go to a workspace and cgemm_parts_kernel adds them in
+// order (the paper's U^T * U, 300 x 100000 x 300, three slices, 27 tiles:
+// 3.53 -> 0.73 ms and 0.013 ms for the sums).
 // K is cut into chunks of KCB K blocks (256 bf16 or 128 tf32 elements): every
 // chunk accumulates into a fresh TMEM set (the sets alternate, so the next
 // chunk's MMAs run while the epilogue drains the previous one) and the
@@ -37,6 +41,8 @@
 // for its own copies in flight, frees its tensor memory and exits.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+
+#include <algorithm>
 
 #include "tp_internal.cuh"
 
@@ -65,6 +71,8 @@ struct TcParams {
   int64_t h, n3;
   int32_t* status;
   int mt, nt;   // output tiles along M and N
+  int splits;       // parts of K a tile is cut into (> 1: zr, zi are partial sums,
+  int64_t s_split;  //   part sp at sp * s_split)
   long long mma_wait_limit;   // the MMA warp's wait for loaded stages (clock64 ticks)
 };
 
@@ -199,10 +207,17 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// First chunk of part sp of a tile's nch accumulation chunks.
+__device__ __forceinline__ int part_begin(int nch, int splits, int sp) {
+  return nch / splits * sp + min(sp, nch % splits);
+}
+
 // Ten warps: two of the four SM sub-partitions hold three of them, and a
 // sub-partition's 16K registers then allow 170 per thread; the epilogue's
 // 128 float32 accumulators fit with 8-column TMEM loads.
-template <bool BF16>
+// PARTS: with K parts (the plain form keeps its shorter loops:
+// 9% of a product of 33 slices of 2000 x 400 x 1500).
+template <bool BF16, bool PARTS>
 __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant__ TcParams p) {
   constexpr int TBK = BF16 ? ROWB / 2 : ROWB / 4;   // K elements per K block
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -226,6 +241,8 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
   const int tiles_per_f = p.mt * p.nt;
   const int64_t ntiles = int64_t(tiles_per_f) * p.h;
   const int nch = (nkb + KCB - 1) / KCB;   // accumulation chunks per tile
+  const int splits = PARTS ? p.splits : 1;   // work item: tile * splits + part
+  const int64_t nitems = ntiles * splits;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -259,11 +276,15 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
     // ---------------- TMA producer: stage ring continues across tiles
     int64_t it = 0;   // global K-block counter of this CTA
     bool ok = true;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+      const int64_t t = item / splits;
+      const int sp = int(item - t * splits);
+      const int c0 = PARTS ? part_begin(nch, splits, sp) : 0;
+      const int c1 = PARTS ? part_begin(nch, splits, sp + 1) : nch;
       const int f = int(t / tiles_per_f);
       const int rem = int(t - int64_t(f) * tiles_per_f);
       const int m0 = (rem / p.nt) * TM, n0 = (rem % p.nt) * TN;
-      for (int kb = 0; kb < nkb; ++kb, ++it) {
+      for (int kb = c0 * KCB; kb < (PARTS ? min(nkb, c1 * KCB) : nkb); ++kb, ++it) {
         const int s = int(it % STAGES);
         const int64_t r = it / STAGES;
         if (r > 0) {
@@ -296,10 +317,14 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
     int64_t ch = 0;   // global chunk counter (accumulator sets alternate per chunk)
     bool ok = true;
     const uint32_t id = BF16 ? IDESC_BF16 : IDESC, idn = BF16 ? IDESC_BF16_NEG : IDESC_NEG;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+      const int64_t t = item / splits;
+      const int sp = int(item - t * splits);
+      const int c0 = PARTS ? part_begin(nch, splits, sp) : 0;
+      const int c1 = PARTS ? part_begin(nch, splits, sp + 1) : nch;
       const int f = int(t / tiles_per_f);
       const bool real_slice = (f == 0) || ((p.n3 % 2 == 0) && f == p.h - 1);
-      for (int c = 0; c < nch && ok; ++c, ++ch) {
+      for (int c = c0; c < c1 && ok; ++c, ++ch) {
         const int b = int(ch & 1);
         const int64_t use = ch >> 1;
         if (use > 0 && !mbar_wait(smem_u32(&acc_empty[b]), uint32_t((use - 1) & 1))) {
@@ -366,19 +391,23 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
     const int half = (warp - 2) >> 2;
     int64_t ch = 0;
     bool stop = false;
-    for (int64_t t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
+    for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x) {
+      const int64_t t = item / splits;
+      const int sp = int(item - t * splits);
       const int f = int(t / tiles_per_f);
       const int rem = int(t - int64_t(f) * tiles_per_f);
       const int64_t m0 = int64_t(rem / p.nt) * TM;
       const int64_t n0 = int64_t(rem % p.nt) * TN + half * EPI_COLS;
       const bool real_slice = (f == 0) || ((p.n3 % 2 == 0) && f == p.h - 1);
+      const int nc =
+          PARTS ? part_begin(nch, splits, sp + 1) - part_begin(nch, splits, sp) : nch;
       float accr[EPI_COLS], acci[EPI_COLS];
 #pragma unroll
       for (int j = 0; j < EPI_COLS; ++j) {
         accr[j] = 0.f;
         acci[j] = 0.f;
       }
-      for (int c = 0; c < nch; ++c, ++ch) {
+      for (int c = 0; c < nc; ++c, ++ch) {
         const int b = int(ch & 1);
         const int64_t use = ch >> 1;
         bool have = mbar_wait(smem_u32(&acc_full[b]), uint32_t(use & 1));
@@ -389,18 +418,18 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
           const uint32_t base = tmem + (uint32_t(q * 32) << 16) + uint32_t(b) * (2 * TN) +
                                 uint32_t(half * EPI_COLS);
 #pragma unroll
-          for (int c0 = 0; c0 < EPI_COLS; c0 += 8) {
+          for (int q0 = 0; q0 < EPI_COLS; q0 += 8) {
             uint32_t vr[8], vi[8];
-            tmem_ld8_nowait(base + uint32_t(c0), vr);
-            if (!real_slice) tmem_ld8_nowait(base + uint32_t(TN + c0), vi);
+            tmem_ld8_nowait(base + uint32_t(q0), vr);
+            if (!real_slice) tmem_ld8_nowait(base + uint32_t(TN + q0), vi);
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               // chunk sums added in float32, round to nearest
-              accr[c0 + j] = c == 0 ? __uint_as_float(vr[j]) : accr[c0 + j] + __uint_as_float(vr[j]);
+              accr[q0 + j] = c == 0 ? __uint_as_float(vr[j]) : accr[q0 + j] + __uint_as_float(vr[j]);
               if (!real_slice)
-                acci[c0 + j] =
-                    c == 0 ? __uint_as_float(vi[j]) : acci[c0 + j] + __uint_as_float(vi[j]);
+                acci[q0 + j] =
+                    c == 0 ? __uint_as_float(vi[j]) : acci[q0 + j] + __uint_as_float(vi[j]);
             }
           }
         }
@@ -416,8 +445,8 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
       if (stop) break;
       const int64_t m = m0 + q * 32 + lane;
       if (m < p.M) {
-        float* zr = p.zr + int64_t(f) * p.sZ;
-        float* zi = p.zi + int64_t(f) * p.sZ;
+        float* zr = p.zr + (PARTS ? int64_t(sp) * p.s_split : 0) + int64_t(f) * p.sZ;
+        float* zi = p.zi + (PARTS ? int64_t(sp) * p.s_split : 0) + int64_t(f) * p.sZ;
 #pragma unroll
         for (int j = 0; j < EPI_COLS; ++j) {
           const int64_t n = n0 + j;
@@ -439,6 +468,29 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
                  "r"(TMEM_COLS)
                  : "memory");
   }
+}
+
+// C = the sum of the K parts of every output (planes of n per part, in order).
+__global__ void __launch_bounds__(256) cgemm_parts_kernel(const float* __restrict__ part, int64_t n,
+                                                          int64_t s_split, int splits,
+                                                          float* __restrict__ out) {
+  for (int64_t e = int64_t(blockIdx.x) * 256 + threadIdx.x; e < n; e += int64_t(gridDim.x) * 256) {
+    float a = part[e];
+    for (int sp = 1; sp < splits; ++sp) a += part[e + sp * s_split];
+    out[e] = a;
+  }
+}
+
+// Parts of K for a product with few output tiles: as many as fill the SMs
+// once, at most one per accumulation chunk.  Sized for GB300's 152 SMs
+// wherever it runs, so that a workspace query needs no device.
+int cgemm_splits(int64_t M, int64_t N, int64_t h, int64_t kcap, int precision) {
+  const int64_t tiles = (M + TM - 1) / TM * ((N + TN - 1) / TN) * h;
+  const int64_t chunk = int64_t(KCB) * ROWB / (precision == TP_BF16X3 ? 2 : 4);
+  const int64_t chunks = (kcap + chunk - 1) / chunk;
+  int64_t s = 152 / (tiles < 1 ? 1 : tiles);
+  if (s > chunks) s = chunks;
+  return s < 2 ? 1 : int(s > 64 ? 64 : s);
 }
 
 // ---------------------------------------------------------------- host side
@@ -483,6 +535,11 @@ int encode_map(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uin
 }
 
 }  // namespace
+
+size_t cgemm_split_floats(int64_t M, int64_t N, int64_t h, int64_t kcap, int precision) {
+  const int s = cgemm_splits(M, N, h, kcap, precision);
+  return s > 1 ? 2 * size_t(s) * size_t(M) * size_t(N) * size_t(h) : 0;
+}
 
 // Operands for the tensor-core path come as split planes: g.ar/g.ai are the
 // hi planes and g.ar_lo/g.ai_lo (likewise b) the lo planes, float (3xTF32) or
@@ -540,17 +597,37 @@ int launch_cgemm_tc(const CGemm& g, cudaStream_t st) {
   p.status = g.status;
   p.mt = int((g.M + TM - 1) / TM);
   p.nt = int((g.N + TN - 1) / TN);
+  // parts of K where the caller gave room for them (and C is contiguous)
+  const int splits = g.split_ws && g.ldc == g.M && g.sC == g.M * g.N
+                         ? cgemm_splits(g.M, g.N, g.h, g.dynK ? g.kcap : g.K, g.precision)
+                         : 1;
+  p.splits = splits;
+  p.s_split = splits > 1 ? g.M * g.N * g.h : 0;
+  if (splits > 1) {
+    p.zr = g.split_ws;
+    p.zi = g.split_ws + int64_t(splits) * p.s_split;
+  }
   p.mma_wait_limit = g.wait_limit > 0 ? g.wait_limit : WAIT_LIMIT;
-  auto kernel = bf16 ? cgemm_tc_kernel<true> : cgemm_tc_kernel<false>;
+  auto kernel = splits > 1 ? (bf16 ? cgemm_tc_kernel<true, true> : cgemm_tc_kernel<false, true>)
+                                     : (bf16 ? cgemm_tc_kernel<true, false> : cgemm_tc_kernel<false, false>);
   TP_SET_SMEM(kernel, SMEM_BYTES);
   const int sms = sm_count();
-  const int64_t ntiles = int64_t(p.mt) * p.nt * g.h;
-  const dim3 grid(unsigned(ntiles < sms ? ntiles : sms));
+  const int64_t nitems = int64_t(p.mt) * p.nt * g.h * splits;
+  const dim3 grid(unsigned(nitems < sms ? nitems : sms));
   {
     KernelScope ks("cgemm_tc", st);
     kernel<<<grid, NTHR, SMEM_BYTES, st>>>(p);
   }
-  return launch_status("cgemm_tc_kernel");
+  int rc = launch_status("cgemm_tc_kernel");
+  if (rc || splits == 1) return rc;
+  const int64_t n = p.s_split;
+  const unsigned blocks = unsigned(std::min<int64_t>((n + 255) / 256, int64_t(sms) * 8));
+  for (int pl = 0; pl < 2; ++pl) {
+    KernelScope ks("cgemm_parts", st);
+    cgemm_parts_kernel<<<blocks, 256, 0, st>>>(pl ? p.zi : p.zr, n, p.s_split, splits,
+                                               pl ? g.ci : g.cr);
+  }
+  return launch_status("cgemm_parts_kernel");
 }
 
 }  // namespace tp

@@ -117,13 +117,16 @@ KernelScope::~KernelScope() {
   if (slot < int(g_prof_recs.size())) cudaEventRecord(g_prof_recs[slot].b, st);
 }
 
-int acquire_workspace(const tp_opts* opts, size_t need, Arena* out) {
+int acquire_workspace(const tp_opts* opts, size_t need, Arena* out, size_t least, bool* lean) {
+  if (lean) *lean = false;
   if (opts && opts->workspace) {
     if ((reinterpret_cast<uintptr_t>(opts->workspace) & 255) != 0) {
       set_error("workspace must be 256-byte aligned");
       return TP_EALIGN;
     }
-    if (opts->workspace_bytes < need) {
+    if (opts->workspace_bytes < need && lean && opts->workspace_bytes >= least) {
+      *lean = true;
+    } else if (opts->workspace_bytes < need) {
       set_error("workspace of %zu bytes is smaller than the %zu this call needs",
                 opts->workspace_bytes, need);
       return TP_EWORKSPACE;

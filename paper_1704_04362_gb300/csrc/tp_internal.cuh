@@ -57,7 +57,11 @@ inline size_t ws_bytes(size_t count, size_t elem) { return (count * elem + 255) 
 
 // Resolves the workspace of a call: opts->workspace when given (checked
 // against `need`), else the library-managed per-device buffer.
-int acquire_workspace(const tp_opts* opts, size_t need, Arena* out);
+// `need` bytes from opts->workspace or the device's own buffer.  With `lean`,
+// a caller's workspace of at least `least` bytes is taken too and *lean set:
+// the call then goes without what only makes it faster.
+int acquire_workspace(const tp_opts* opts, size_t need, Arena* out, size_t least = 0,
+                      bool* lean = nullptr);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 inline int64_t half_len(int64_t n3) { return n3 / 2 + 1; }
@@ -114,7 +118,12 @@ struct CGemm {
   // FP32 path only: B_k(kk, n) = conj(b[k*sB + n + ldb*kk]) (B given as its
   // conjugate transpose)
   int b_conj_trans = 0;
+  // tensor-core path: room for the partial sums of a K cut into parts
+  // (cgemm_split_floats()), or null: K is not cut
+  float* split_ws = nullptr;
 };
+// Floats a tensor-core product wants for its K parts (0: it is not cut).
+size_t cgemm_split_floats(int64_t M, int64_t N, int64_t h, int64_t kcap, int precision);
 int launch_cgemm(const CGemm& g, cudaStream_t st);
 
 // Slice norms (squared, float64).  Lateral: out[j] = sum over (i,t) of X(i,j,t)^2.
