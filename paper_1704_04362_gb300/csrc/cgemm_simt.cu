@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(S::NT) cgemm_simt_kernel(const __grid_constant
   extern __shared__ __align__(16) float cg_sm[];
   const int64_t K = g.dynK ? *g.dynK : g.K;
   for (int64_t f = blockIdx.z; f < g.h; f += gridDim.z) {
+    if (g.only && g.only[f] != g.only_val) continue;
     const bool real = (f == 0) || ((g.n3 % 2 == 0) && f == g.h - 1);
     if (real) cgemm_tile<S, true, CONJ>(g, f, K, cg_sm);
     else cgemm_tile<S, false, CONJ>(g, f, K, cg_sm);

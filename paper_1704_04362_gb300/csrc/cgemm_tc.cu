@@ -73,6 +73,8 @@ struct TcParams {
   int mt, nt;   // output tiles along M and N
   int splits;       // parts of K a tile is cut into (> 1: zr, zi are partial sums,
   int64_t s_split;  //   part sp at sp * s_split)
+  const int* only;   // per slice, or null: slices with only[f] != only_val are skipped
+  int only_val;
   long long mma_wait_limit;   // the MMA warp's wait for loaded stages (clock64 ticks)
 };
 
@@ -215,7 +217,7 @@ __device__ __forceinline__ int part_begin(int nch, int splits, int sp) {
 // Ten warps: two of the four SM sub-partitions hold three of them, and a
 // sub-partition's 16K registers then allow 170 per thread; the epilogue's
 // 128 float32 accumulators fit with 8-column TMEM loads.
-// PARTS: with K parts (the plain form keeps its shorter loops:
+// PARTS: with K parts or skipped slices (the plain form keeps its shorter loops:
 // 9% of a product of 33 slices of 2000 x 400 x 1500).
 template <bool BF16, bool PARTS>
 __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant__ TcParams p) {
@@ -282,6 +284,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
       const int c0 = PARTS ? part_begin(nch, splits, sp) : 0;
       const int c1 = PARTS ? part_begin(nch, splits, sp + 1) : nch;
       const int f = int(t / tiles_per_f);
+      if (PARTS && p.only && p.only[f] != p.only_val) continue;
       const int rem = int(t - int64_t(f) * tiles_per_f);
       const int m0 = (rem / p.nt) * TM, n0 = (rem % p.nt) * TN;
       for (int kb = c0 * KCB; kb < (PARTS ? min(nkb, c1 * KCB) : nkb); ++kb, ++it) {
@@ -323,6 +326,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
       const int c0 = PARTS ? part_begin(nch, splits, sp) : 0;
       const int c1 = PARTS ? part_begin(nch, splits, sp + 1) : nch;
       const int f = int(t / tiles_per_f);
+      if (PARTS && p.only && p.only[f] != p.only_val) continue;
       const bool real_slice = (f == 0) || ((p.n3 % 2 == 0) && f == p.h - 1);
       for (int c = c0; c < c1 && ok; ++c, ++ch) {
         const int b = int(ch & 1);
@@ -395,6 +399,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
       const int64_t t = item / splits;
       const int sp = int(item - t * splits);
       const int f = int(t / tiles_per_f);
+      if (PARTS && p.only && p.only[f] != p.only_val) continue;
       const int rem = int(t - int64_t(f) * tiles_per_f);
       const int64_t m0 = int64_t(rem / p.nt) * TM;
       const int64_t n0 = int64_t(rem % p.nt) * TN + half * EPI_COLS;
@@ -598,7 +603,7 @@ int launch_cgemm_tc(const CGemm& g, cudaStream_t st) {
   p.mt = int((g.M + TM - 1) / TM);
   p.nt = int((g.N + TN - 1) / TN);
   // parts of K where the caller gave room for them (and C is contiguous)
-  const int splits = g.split_ws && g.ldc == g.M && g.sC == g.M * g.N
+  const int splits = g.split_ws && !g.only && g.ldc == g.M && g.sC == g.M * g.N
                          ? cgemm_splits(g.M, g.N, g.h, g.dynK ? g.kcap : g.K, g.precision)
                          : 1;
   p.splits = splits;
@@ -607,8 +612,10 @@ int launch_cgemm_tc(const CGemm& g, cudaStream_t st) {
     p.zr = g.split_ws;
     p.zi = g.split_ws + int64_t(splits) * p.s_split;
   }
+  p.only = g.only;
+  p.only_val = g.only_val;
   p.mma_wait_limit = g.wait_limit > 0 ? g.wait_limit : WAIT_LIMIT;
-  auto kernel = splits > 1 ? (bf16 ? cgemm_tc_kernel<true, true> : cgemm_tc_kernel<false, true>)
+  auto kernel = splits > 1 || g.only ? (bf16 ? cgemm_tc_kernel<true, true> : cgemm_tc_kernel<false, true>)
                                      : (bf16 ? cgemm_tc_kernel<true, false> : cgemm_tc_kernel<false, false>);
   TP_SET_SMEM(kernel, SMEM_BYTES);
   const int sms = sm_count();

@@ -54,7 +54,9 @@ template <int RPL>
 __global__ void __launch_bounds__(JB_THREADS) jacobi_blocked_kernel(
     float* __restrict__ g_re, float* __restrict__ g_im, int64_t sG, float* __restrict__ v_re,
     float* __restrict__ v_im, int64_t sV, float* __restrict__ sig, int p, int q, int max_sweeps,
-    const int* __restrict__ real_flags, int32_t* __restrict__ status, int init_v) {
+    const int* __restrict__ real_flags, int32_t* __restrict__ status, int init_v,
+    const int* __restrict__ skip) {
+  if (skip && skip[blockIdx.x]) return;   // this slice needs no vectors
   extern __shared__ __align__(16) float jb_smem[];
   // staged columns of G at stride ld (the register path's 32 RPL >= p rows:
   // its lanes move 4 consecutive rows with one 16-byte access and the zero
@@ -446,13 +448,14 @@ size_t jb_smem_bytes(int p) {
 template <int RPL>
 int jb_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi, int64_t sV, float* sig,
               int p, int q, int batch, int max_sweeps, const int* real_flags, int32_t* status,
-              bool init_v, cudaStream_t st) {
+              bool init_v, const int* skip, cudaStream_t st) {
   const size_t smem = jb_smem_bytes(RPL > 0 ? 32 * RPL : p);
   TP_SET_SMEM(jacobi_blocked_kernel<RPL>, smem);
   {
     KernelScope ks("jacobi_blocked", st);
     jacobi_blocked_kernel<RPL><<<unsigned(batch), JB_THREADS, smem, st>>>(
-        gr, gi, sG, vr, vi, sV, sig, p, q, max_sweeps, real_flags, status, init_v ? 1 : 0);
+        gr, gi, sG, vr, vi, sV, sig, p, q, max_sweeps, real_flags, status, init_v ? 1 : 0,
+        skip);
   }
   return launch_status("jacobi_blocked_kernel");
 }
@@ -467,28 +470,29 @@ bool jacobi_blocked_applies(int p, int q) {
 }
 
 // float32 blocked one-sided Jacobi from V = I (init_v) or from the given V
-// (then G must be the work matrix times that V); G is left rotated.
+// (then G must be the work matrix times that V); G is left rotated.  Slices
+// with skip[b] != 0 (skip may be null) are left alone.
 int jacobi_float_blocked_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi,
                                 int64_t sV, float* sig, int p, int q, int batch, int max_sweeps,
                                 const int* real_flags, int32_t* status, bool init_v,
-                                cudaStream_t st) {
+                                const int* skip, cudaStream_t st) {
   if (batch <= 0 || q <= 0) return TP_OK;
   // the register form's rows come in steps of 128 (the zero rows past p
   // cost the same arithmetic as data rows)
   if (p <= 128)
     return jb_launch<4>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags, status,
-                        init_v, st);
+                        init_v, skip, st);
   if (p <= 256)
     return jb_launch<8>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags, status,
-                        init_v, st);
+                        init_v, skip, st);
   if (p <= 384)
     return jb_launch<12>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags, status,
-                         init_v, st);
+                         init_v, skip, st);
   if (p <= 512)
     return jb_launch<16>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags, status,
-                         init_v, st);
+                         init_v, skip, st);
   return jb_launch<0>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags, status,
-                      init_v, st);
+                      init_v, skip, st);
 }
 
 }  // namespace tp

@@ -68,8 +68,10 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(T* g_re, T* g_im, i
                                                              T* v_im, int64_t sV, T* sig, int p,
                                                              int q, int max_sweeps,
                                                              const int* real_flags,
-                                                             int32_t* status, int flags) {
+                                                             int32_t* status, int flags,
+                                                             const int* skip) {
   extern __shared__ __align__(16) unsigned char jac_smem[];
+  if (skip && skip[blockIdx.x]) return;   // this slice needs no vectors
   const int64_t b = blockIdx.x;
   T* const gGr = g_re + b * sG;
   T* const gGi = g_im + b * sG;
@@ -367,11 +369,12 @@ template <class T, bool S>
 __global__ void __cluster_dims__(JPC, 1, 1) __launch_bounds__(JPC_THREADS)
     jacobi_cluster_kernel(T* g_re, T* g_im, int64_t sG, T* v_re, T* v_im, int64_t sV, T* nrm_ws,
                           T* sig, int p, int q, int max_sweeps, const int* real_flags,
-                          int32_t* status, int flags) {
+                          int32_t* status, int flags, const int* skip) {
   extern __shared__ __align__(16) unsigned char jpc_smem[];
   constexpr bool keep = sizeof(T) == 8;
   const int c = int(jpc_rank());
   const int64_t b = blockIdx.x / JPC;
+  if (skip && skip[b]) return;   // the whole cluster: this slice needs no vectors
   T* const Gr = g_re + b * sG;
   T* const Gi = g_im + b * sG;
   T* const Vr = v_re + b * sV;
@@ -736,7 +739,7 @@ size_t jacobi_smem(int p, int q) {
 template <class T>
 int jacobi_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T* sig, int p, int q,
                   int batch, int max_sweeps, const int* real_flags, int32_t* status, int flags,
-                  cudaStream_t st) {
+                  cudaStream_t st, const int* skip = nullptr) {
   if (batch <= 0 || q <= 0) return TP_OK;
   if (q > JAC_MAX_Q) {
     set_error("jacobi: %d columns, more than %d", q, JAC_MAX_Q);
@@ -750,7 +753,7 @@ int jacobi_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T* sig, in
   {
     KernelScope ks(sizeof(T) == 4 ? "jacobi_f32" : "jacobi_svd", st);
     jacobi_kernel<T><<<unsigned(batch), SVD_THREADS, smem, st>>>(
-        gr, gi, sG, vr, vi, sV, sig, p, q, max_sweeps, real_flags, status, flags);
+        gr, gi, sG, vr, vi, sV, sig, p, q, max_sweeps, real_flags, status, flags, skip);
   }
   return launch_status("jacobi_kernel");
 }
@@ -791,7 +794,8 @@ bool use_cluster(int q, int batch) {
 template <class T>
 int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T* nrm, T* sig,
                           int p, int q, int batch, int max_sweeps, const int* real_flags,
-                          int32_t* status, int flags, cudaStream_t st) {
+                          int32_t* status, int flags, cudaStream_t st,
+                          const int* skip = nullptr) {
   if (batch <= 0 || q <= 0) return TP_OK;
   const size_t smem = jacobi_cluster_smem<T>(p, q);
   const unsigned grid = unsigned(batch) * JPC;
@@ -802,10 +806,10 @@ int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T*
                                  "jacobi_cluster_kernel"))
         return rc;
       jacobi_cluster_kernel<T, true><<<grid, JPC_THREADS, smem, st>>>(
-          gr, gi, sG, vr, vi, sV, nrm, sig, p, q, max_sweeps, real_flags, status, flags);
+          gr, gi, sG, vr, vi, sV, nrm, sig, p, q, max_sweeps, real_flags, status, flags, skip);
     } else {
       jacobi_cluster_kernel<T, false><<<grid, JPC_THREADS, 0, st>>>(
-          gr, gi, sG, vr, vi, sV, nrm, sig, p, q, max_sweeps, real_flags, status, flags);
+          gr, gi, sG, vr, vi, sV, nrm, sig, p, q, max_sweeps, real_flags, status, flags, skip);
     }
   }
   return launch_status("jacobi_cluster_kernel");
@@ -815,11 +819,13 @@ int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T*
 
 // float32 one-sided Jacobi from V = I (init_v) or from the given V (then G
 // must be the work matrix times that V); G is left rotated, not normalised.
+// Slices with skip[b] != 0 (skip may be null) are left alone.
 int jacobi_float_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi, int64_t sV,
                         float* sig, int p, int q, int batch, int max_sweeps,
-                        const int* real_flags, int32_t* status, bool init_v, cudaStream_t st) {
+                        const int* real_flags, int32_t* status, bool init_v, const int* skip,
+                        cudaStream_t st) {
   return jacobi_launch<float>(gr, gi, sG, vr, vi, sV, sig, p, q, batch, max_sweeps, real_flags,
-                              status, init_v ? JAC_INIT_V : 0, st);
+                              status, init_v ? JAC_INIT_V : 0, st, skip);
 }
 
 // Whether jacobi_float_cluster_launch takes a batch of p x q slices (fewer
@@ -830,9 +836,10 @@ bool jacobi_cluster_applies(int q, int batch) { return use_cluster(q, batch); }
 int jacobi_float_cluster_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi,
                                 int64_t sV, float* sig, int p, int q, int batch, int max_sweeps,
                                 const int* real_flags, int32_t* status, bool init_v,
-                                cudaStream_t st) {
+                                const int* skip, cudaStream_t st) {
   return jacobi_cluster_launch<float>(gr, gi, sG, vr, vi, sV, nullptr, sig, p, q, batch,
-                                      max_sweeps, real_flags, status, init_v ? JAC_INIT_V : 0, st);
+                                      max_sweeps, real_flags, status, init_v ? JAC_INIT_V : 0, st,
+                                      skip);
 }
 
 // C_b = op(A_b) B_b in float64 from float32 planes (see zgemm64_kernel).

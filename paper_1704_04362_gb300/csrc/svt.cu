@@ -30,23 +30,25 @@
 #include <vector>
 
 #include "dft_common.cuh"
+#include "svt_top.cuh"
 #include "tp_internal.cuh"
 
 namespace tp {
 
 int jacobi_float_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi, int64_t sV,
                         float* sig, int p, int q, int batch, int max_sweeps,
-                        const int* real_flags, int32_t* status, bool init_v, cudaStream_t st);
+                        const int* real_flags, int32_t* status, bool init_v, const int* skip,
+                        cudaStream_t st);
 bool jacobi_blocked_applies(int p, int q);
 bool jacobi_cluster_applies(int q, int batch);
 int jacobi_float_cluster_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi,
                                 int64_t sV, float* sig, int p, int q, int batch, int max_sweeps,
                                 const int* real_flags, int32_t* status, bool init_v,
-                                cudaStream_t st);
+                                const int* skip, cudaStream_t st);
 int jacobi_float_blocked_launch(float* gr, float* gi, int64_t sG, float* vr, float* vi,
                                 int64_t sV, float* sig, int p, int q, int batch, int max_sweeps,
                                 const int* real_flags, int32_t* status, bool init_v,
-                                cudaStream_t st);
+                                const int* skip, cudaStream_t st);
 // Slices too large for the shared-memory Jacobi take the blocked one
 // (jacobi_blocked.cu); -DTP_SVT_BLOCKED=0 keeps them on the global-memory form.
 #ifndef TP_SVT_BLOCKED
@@ -121,6 +123,31 @@ __global__ void to_work_kernel(const float* __restrict__ xr, const float* __rest
   }
 }
 
+// Conjugate transpose of every slice: out (n2 x n1) = M_hat_k^H, 32 x 32 tiles
+// through shared memory.
+__global__ void conj_transpose_work_kernel(const float* __restrict__ xr,
+                                           const float* __restrict__ xi, int64_t n1, int64_t n2,
+                                           float* __restrict__ outr, float* __restrict__ outi) {
+  __shared__ float tr[32][33], ti[32][33];
+  const int64_t o = int64_t(blockIdx.z) * n1 * n2;
+  const int64_t i0 = int64_t(blockIdx.x) * 32, j0 = int64_t(blockIdx.y) * 32;
+  for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
+    const int64_t i = i0 + threadIdx.x, j = j0 + dy;
+    if (i < n1 && j < n2) {
+      tr[dy][threadIdx.x] = xr[o + i + n1 * j];
+      ti[dy][threadIdx.x] = xi[o + i + n1 * j];
+    }
+  }
+  __syncthreads();
+  for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
+    const int64_t j = j0 + threadIdx.x, i = i0 + dy;
+    if (i < n1 && j < n2) {
+      outr[o + j + n2 * i] = tr[threadIdx.x][dy];
+      outi[o + j + n2 * i] = -ti[threadIdx.x][dy];
+    }
+  }
+}
+
 // Shrink factors of every slice from V (q x q) and H = W V (p x q; W the
 // work matrix): with n_j = ||v_j|| and s_j = ||h_j|| / n_j (norms accumulated
 // in float64), c_j = max(s_j - tau, 0) / (s_j n_j^2), so that the shrunk
@@ -133,9 +160,11 @@ __global__ void svt_coef_kernel(const float* __restrict__ hr, const float* __res
                                 const float* __restrict__ vr,
                                 const float* __restrict__ vi, int64_t sV, int p, int q,
                                 const double* __restrict__ mu, bool transpose,
-                                float* __restrict__ outr, float* __restrict__ outi) {
+                                float* __restrict__ outr, float* __restrict__ outi,
+                                const int* __restrict__ skip) {
   extern __shared__ float coef[];   // q factors c_j
   const int64_t f = blockIdx.x;
+  if (skip && skip[f]) return;
   const double tau = 1.0 / *mu;
   const float* Hr = hr + f * sH;
   const float* Hi = hi + f * sH;
@@ -179,11 +208,13 @@ __global__ void svt_split_kernel(const float* __restrict__ sr, const float* __re
                                  int64_t rows, int64_t cols, int64_t ld_src, int64_t s_src,
                                  int64_t h, int64_t ld_dst, int64_t s_dst, int conj, int bf16,
                                  float* __restrict__ p0, float* __restrict__ p1,
-                                 float* __restrict__ p2, float* __restrict__ p3) {
+                                 float* __restrict__ p2, float* __restrict__ p3,
+                                 const int* __restrict__ skip) {
   const int64_t per = ld_dst * cols, total = per * h;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
        e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t f = e / per, rem = e - f * per;
+    if (skip && skip[f]) continue;
     const int64_t c = rem / ld_dst, r = rem - c * ld_dst;
     float vr = 0.f, vi = 0.f;
     if (r < rows) {
@@ -202,9 +233,11 @@ __global__ void svt_split_kernel(const float* __restrict__ sr, const float* __re
 __global__ void svt_split_t_kernel(const float* __restrict__ sr, const float* __restrict__ si,
                                    int64_t rows, int64_t cols, int64_t ld_dst, int64_t s_dst,
                                    int bf16, float* __restrict__ p0, float* __restrict__ p1,
-                                   float* __restrict__ p2, float* __restrict__ p3) {
+                                   float* __restrict__ p2, float* __restrict__ p3,
+                                   const int* __restrict__ skip) {
   __shared__ float tr[32][33], ti[32][33];
   const int64_t f = blockIdx.z;
+  if (skip && skip[f]) return;
   const int64_t r0 = int64_t(blockIdx.x) * 32, c0 = int64_t(blockIdx.y) * 32;
   const float* xr = sr + f * rows * cols;
   const float* xi = si + f * rows * cols;
@@ -244,6 +277,10 @@ int64_t svt_ld(int64_t k, int prec) {
 }
 bool svt_tc(int prec) { return prec == TP_TF32X3 || prec == TP_BF16X3; }
 
+size_t svt_top_bytes(int64_t n1, int64_t n2, int64_t n3) {
+  return svt_top_ws(n1 < n2 ? n1 : n2, size_t(half_len(n3)));
+}
+
 size_t svt_ws(int64_t n1, int64_t n2, int64_t n3, int prec) {
   const size_t h = size_t(half_len(n3));
   const size_t p = size_t(n1 > n2 ? n1 : n2), q = size_t(n1 < n2 ? n1 : n2);
@@ -258,7 +295,8 @@ size_t svt_ws(int64_t n1, int64_t n2, int64_t n3, int prec) {
          + 2 * ws_bytes(q * q * h, 4)         // V
          + 2 * ws_bytes(p * q * h, 4)         // work matrix W
          + 2 * ws_bytes(p * q * h, 4)         // H = W V
-         + ws_bytes(q * h, 4) + ws_bytes(h, 4);
+         + ws_bytes(q * h, 4) + ws_bytes(h, 4) +
+         svt_top_bytes(n1, n2, n3);        // kept vectors and flags of svt_top.cu
 }
 
 // One tensor of a completion run: its ADMM state (caller's buffers) and its
@@ -279,13 +317,16 @@ struct SvtTensor {
   int prec;
   int64_t lq;
   float *WP[4], *HP[4], *VP[4], *BP[4];
+  // sizes that svt_top.cu takes first: its state, and whether it is used
+  SvtTopArgs top;
+  bool use_top = false;
   // a lone tensor (not one of a batch sharing the GPU): its Jacobi may spread
   // each slice over a thread-block cluster when the slices are fewer than SMs
   bool alone = false;
 };
 
 SvtTensor svt_carve(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int64_t n3,
-                    float* L, float* E, float* Y, double* mu, Arena& ws, int prec) {
+                    float* L, float* E, float* Y, double* mu, Arena& ws, int prec, bool lean) {
   SvtTensor t{};
   t.prec = prec;
   t.X = X;
@@ -315,6 +356,24 @@ SvtTensor svt_carve(const float* X, const uint8_t* mask, int64_t n1, int64_t n2,
   t.Hi = ws.take<float>(pq * h);
   t.sig = ws.take<float>(size_t(t.q) * h);
   t.flags = ws.take<int>(h);
+  t.use_top = svt_top_applies(t.q) && !lean;
+  if (t.use_top) {
+    SvtTopArgs& a = t.top;
+    a.gr = t.Gr;
+    a.gi = t.Gi;
+    a.sG = t.p * t.q;
+    a.hr = t.Hr;
+    a.hi = t.Hi;
+    a.xr = ws.take<float>(size_t(t.q) * SVT_TOP_L * h);
+    a.xi = ws.take<float>(size_t(t.q) * SVT_TOP_L * h);
+    a.mu = mu;
+    a.attempt = ws.take<int>(h);
+    a.fast = ws.take<int>(h);
+    a.wait = ws.take<int>(h);
+    a.edge = ws.take<float>(h);
+    a.above = ws.take<unsigned>(h);
+    a.q = int(t.q);
+  }
   t.lq = svt_ld(t.q, prec);
   if (svt_tc(prec)) {
     const size_t lq = size_t(t.lq);
@@ -331,29 +390,70 @@ SvtTensor svt_carve(const float* X, const uint8_t* mask, int64_t n1, int64_t n2,
   return t;
 }
 
+// Flags of a run's real slices and, where svt_top.cu is used, its state and
+// V = I for the Jacobi (with V's split planes in the split forms).
 int svt_init(const SvtTensor& t, cudaStream_t st) {
   {
     KernelScope ks("svt_flags", st);
     flags_kernel<<<unsigned((t.h + 255) / 256), 256, 0, st>>>(t.flags, t.h, t.n3);
   }
-  return launch_status("svt_flags");
+  int rc = launch_status("svt_flags");
+  if (rc || !t.use_top) return rc;
+  if ((rc = svt_top_init(t.top, t.h, t.Vr, t.Vi, st))) return rc;
+  if (!svt_tc(t.prec)) return TP_OK;
+  {
+    KernelScope ks("svt_split", st);
+    svt_split_kernel<<<grid_n(t.lq * t.q * t.h), 256, 0, st>>>(
+        t.Vr, t.Vi, t.q, t.q, t.q, t.q * t.q, t.h, t.lq, t.lq * t.q, 0, t.prec == TP_BF16X3 ? 1 : 0,
+        t.VP[0], t.VP[1], t.VP[2], t.VP[3], nullptr);
+  }
+  return launch_status("svt_split_kernel");
 }
 
-// One ADMM iteration of one tensor on stream st.  warm: start the Jacobi from
-// the V left by the previous iteration of this tensor.
-int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int sweeps,
-                  int32_t* status, cudaStream_t st) {
+// L_hat = SVT(M_hat) of one tensor, M_hat and L_hat in t.Mr, t.Mi.  warm: start
+// the Jacobi from the V left by the previous iteration of this tensor (always
+// so where svt_top.cu is used: its V starts as I).
+int svt_shrink(const SvtTensor& t, bool warm, int sweeps, int32_t* status, cudaStream_t st) {
   int rc;
-  const int64_t n = t.n1 * t.n2 * t.n3, n12 = t.n1 * t.n2;
+  const int64_t n12 = t.n1 * t.n2;
   const int64_t p = t.p, q = t.q, h = t.h;
-  {
-    KernelScope ks("admm_pre", st);
-    admm_pre_kernel<<<grid_n(n), 256, 0, st>>>(t.X, t.mask, t.E, t.Y, t.mu, n, t.M);
-  }
-  DftGather gm{t.M, n12, 1, 1, 0, n12, nullptr, nullptr, nullptr, 0, t.n3, t.Mr, t.Mi,
-               n12, n12, nullptr, nullptr, 0};
-  if ((rc = launch_rdft(gm, st))) return rc;
-  {   // work matrix W (kept in K), and G = W for a cold start
+  const bool top = t.use_top;
+  const int* skip = nullptr;   // slices that svt_top.cu has thresholded
+  const float *Wr = t.Kr, *Wi = t.Ki;   // the work matrix W = M_hat or M_hat^H (p x q)
+  if (top) {
+    // K = M_hat^H; W is whichever of M_hat and K is p x q, the other is W^H
+    {
+      KernelScope ks("svt_work", st);
+      conj_transpose_work_kernel<<<dim3(unsigned((t.n1 + 31) / 32), unsigned((t.n2 + 31) / 32),
+                                        unsigned(h)),
+                                   dim3(32, 8), 0, st>>>(t.Mr, t.Mi, t.n1, t.n2, t.Kr, t.Ki);
+    }
+    if ((rc = launch_status("svt_work"))) return rc;
+    if (!t.transpose) {
+      Wr = t.Mr;
+      Wi = t.Mi;
+    }
+    const float* Ar = t.transpose ? t.Mr : t.Kr;
+    const float* Ai = t.transpose ? t.Mi : t.Ki;
+    // Gram W^H W of the slices that try
+    CGemm gg{Ar, Ai, Wr, Wi, t.Gr, t.Gi, q, q, p, nullptr, q, p, q, p * q, p * q, p * q, h, t.n3,
+             TP_FP32, nullptr, nullptr, nullptr, nullptr, p, status};
+    gg.only = t.top.attempt;
+    gg.only_val = 1;
+    if ((rc = launch_cgemm(gg, st))) return rc;
+    if ((rc = svt_top_launch(t.top, h, st))) return rc;
+    // the thresholded ones: H = W X, the shrink factors, the rebuild
+    CGemm gx{Wr, Wi, t.top.xr, t.top.xi, t.Hr, t.Hi, p, SVT_TOP_L, q, nullptr, p, SVT_TOP_L, p,
+             p * q, q * SVT_TOP_L, p * q, h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q,
+             status};
+    gx.b_conj_trans = 1;
+    gx.only = t.top.fast;
+    gx.only_val = 1;
+    if ((rc = launch_cgemm(gx, st))) return rc;
+    if ((rc = svt_top_coef(t.top, h, t.Hr, t.Hi, p, t.transpose, st))) return rc;
+    skip = t.top.fast;
+    warm = true;
+  } else {   // work matrix W (kept in K), and G = W for a cold start
     KernelScope ks("svt_work", st);
     to_work_kernel<<<grid_n(n12 * h), 256, 0, st>>>(t.Mr, t.Mi, t.n1, t.n2, h, t.transpose, t.Kr,
                                                     t.Ki, warm ? nullptr : t.Gr,
@@ -362,13 +462,19 @@ int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int 
   const bool tc = svt_tc(t.prec);
   const int bf = t.prec == TP_BF16X3 ? 1 : 0;
   const int64_t lq = t.lq;
+  // the slices left to the Jacobi
+  auto rest = [&](CGemm& g) {
+    g.only = skip;
+    g.only_val = 0;
+    return launch_cgemm(g, st);
+  };
   // tensor-core GEMM C = A B over the h slices, A (M x K) and B (K x N) split
   // planes stored K-major with leading dimension lq, C column-major (ldc)
   auto gemm_tc = [&](float* const* A, float* const* B, float* cr, float* ci, int64_t M,
                      int64_t N, int64_t ldc) {
     CGemm g{A[0], A[2], B[0], B[2], cr, ci, M, N, q, nullptr, lq, lq, ldc, lq * M, lq * N,
             M * N, h, t.n3, t.prec, A[1], A[3], B[1], B[3], lq, status};
-    return launch_cgemm(g, st);
+    return rest(g);
   };
   auto split = [&](const float* sr, const float* si, int64_t rows, int64_t cols, int conj,
                    float* const* P) {
@@ -376,7 +482,7 @@ int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int 
       KernelScope ks("svt_split", st);
       svt_split_kernel<<<grid_n(lq * cols * h), 256, 0, st>>>(
           sr, si, rows, cols, rows, rows * cols, h, lq, lq * cols, conj, bf, P[0], P[1], P[2],
-          P[3]);
+          P[3], skip);
     }
     return launch_status("svt_split_kernel");
   };
@@ -388,29 +494,45 @@ int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int 
       svt_split_t_kernel<<<dim3(unsigned((rows + 31) / 32), unsigned((lq + 31) / 32),
                                 unsigned(h)),
                            dim3(32, 8), 0, st>>>(sr, si, rows, cols, lq, lq * rows, bf, P[0],
-                                                 P[1], P[2], P[3]);
+                                                 P[1], P[2], P[3], skip);
     }
     return launch_status("svt_split_t_kernel");
   };
-  if (tc && (rc = split_t(t.Kr, t.Ki, p, q, t.WP))) return rc;   // W, row-major
+  if (tc && (rc = split_t(Wr, Wi, p, q, t.WP))) return rc;   // W, row-major
+  if (top) {   // rebuild of the thresholded slices: their operands are in H and G
+    if (!t.transpose) {   // slice (p x q) = H (D X^H)
+      CGemm g{t.Hr, t.Hi, t.Gr, t.Gi, t.Mr, t.Mi, p, q, SVT_TOP_L, nullptr, p, SVT_TOP_L, p, p * q,
+              p * q, p * q, h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, SVT_TOP_L, status};
+      g.only = t.top.fast;
+      g.only_val = 1;
+      if ((rc = launch_cgemm(g, st))) return rc;
+    } else {              // slice (q x p) = (X D) H^H
+      CGemm g{t.Gr, t.Gi, t.Hr, t.Hi, t.Mr, t.Mi, q, p, SVT_TOP_L, nullptr, q, p, q, p * q, p * q,
+              q * p, h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, SVT_TOP_L, status};
+      g.b_conj_trans = 1;
+      g.only = t.top.fast;
+      g.only_val = 1;
+      if ((rc = launch_cgemm(g, st))) return rc;
+    }
+  }
   if (warm) {   // G = W V_prev
     if (tc) {
       if ((rc = gemm_tc(t.WP, t.VP, t.Gr, t.Gi, p, q, p))) return rc;
     } else {
-      CGemm gw{t.Kr, t.Ki, t.Vr, t.Vi, t.Gr, t.Gi, p, q, q, nullptr, p, q, p, p * q, q * q, p * q,
+      CGemm gw{Wr, Wi, t.Vr, t.Vi, t.Gr, t.Gi, p, q, q, nullptr, p, q, p, p * q, q * q, p * q,
                h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q, status};
-      if ((rc = launch_cgemm(gw, st))) return rc;
+      if ((rc = rest(gw))) return rc;
     }
   }
   if (t.alone && jacobi_cluster_applies(int(q), int(h)))
     rc = jacobi_float_cluster_launch(t.Gr, t.Gi, p * q, t.Vr, t.Vi, q * q, t.sig, int(p), int(q),
-                                     int(h), sweeps, t.flags, status, !warm, st);
+                                     int(h), sweeps, t.flags, status, !warm, skip, st);
   else if (TP_SVT_BLOCKED && jacobi_blocked_applies(int(p), int(q)))
     rc = jacobi_float_blocked_launch(t.Gr, t.Gi, p * q, t.Vr, t.Vi, q * q, t.sig, int(p), int(q),
-                                     int(h), sweeps, t.flags, status, !warm, st);
+                                     int(h), sweeps, t.flags, status, !warm, skip, st);
   else
     rc = jacobi_float_launch(t.Gr, t.Gi, p * q, t.Vr, t.Vi, q * q, t.sig, int(p), int(q),
-                             int(h), sweeps, t.flags, status, !warm, st);
+                             int(h), sweeps, t.flags, status, !warm, skip, st);
   if (rc) return rc;
   if (tc) {
     // V's planes (also V_prev of the next iteration's G = W V_prev), then
@@ -418,36 +540,52 @@ int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int 
     if ((rc = split(t.Vr, t.Vi, q, q, 0, t.VP))) return rc;
     if ((rc = gemm_tc(t.VP, t.WP, t.Hr, t.Hi, q, p, q))) return rc;
   } else {   // H = W V from the unrotated work matrix
-    CGemm gh{t.Kr, t.Ki, t.Vr, t.Vi, t.Hr, t.Hi, p, q, q, nullptr, p, q, p, p * q, q * q, p * q,
+    CGemm gh{Wr, Wi, t.Vr, t.Vi, t.Hr, t.Hi, p, q, q, nullptr, p, q, p, p * q, q * q, p * q,
              h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q, status};
-    if ((rc = launch_cgemm(gh, st))) return rc;
+    if ((rc = rest(gh))) return rc;
   }
   {   // shrink factors into the small operand (in G, free after the Jacobi)
     KernelScope ks("svt_coef", st);
     svt_coef_kernel<<<unsigned(h), 256, size_t(q) * sizeof(float), st>>>(
         t.Hr, t.Hi, p * q, tc ? q : 1, tc ? 1 : p, t.Vr, t.Vi, q * q, int(p), int(q), t.mu,
-        t.transpose, t.Gr, t.Gi);
+        t.transpose, t.Gr, t.Gi, skip);
   }
   if (tc) {
     if (!t.transpose) {   // slice (p x q) = H (D V^H)
       if ((rc = split(t.Hr, t.Hi, q, p, 0, t.HP))) return rc;     // H row-major
       if ((rc = split(t.Gr, t.Gi, q, q, 0, t.BP))) return rc;     // D V^H column-major
-      if ((rc = gemm_tc(t.HP, t.BP, t.Mr, t.Mi, p, q, p))) return rc;
-    } else {              // slice (q x p) = (V D) H^H
-      if ((rc = split(t.Hr, t.Hi, q, p, 1, t.HP))) return rc;     // conj(H) row-major
-      if ((rc = split_t(t.Gr, t.Gi, q, q, t.BP))) return rc;      // V D row-major
-      if ((rc = gemm_tc(t.BP, t.HP, t.Mr, t.Mi, q, p, q))) return rc;
+      return gemm_tc(t.HP, t.BP, t.Mr, t.Mi, p, q, p);
     }
-  } else if (!t.transpose) {   // slice = H (D V^H): n1 x n2 = p x q
+    // slice (q x p) = (V D) H^H
+    if ((rc = split(t.Hr, t.Hi, q, p, 1, t.HP))) return rc;     // conj(H) row-major
+    if ((rc = split_t(t.Gr, t.Gi, q, q, t.BP))) return rc;      // V D row-major
+    return gemm_tc(t.BP, t.HP, t.Mr, t.Mi, q, p, q);
+  }
+  if (!t.transpose) {   // slice = H (D V^H): n1 x n2 = p x q
     CGemm gr{t.Hr, t.Hi, t.Gr, t.Gi, t.Mr, t.Mi, p, q, q, nullptr, p, q, p, p * q, q * q, p * q,
              h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q, status};
-    if ((rc = launch_cgemm(gr, st))) return rc;
-  } else {              // slice = (V D) H^H: n1 x n2 = q x p
-    CGemm gr{t.Gr, t.Gi, t.Hr, t.Hi, t.Mr, t.Mi, q, p, q, nullptr, q, p, q, q * q, p * q, q * p,
-             h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q, status};
-    gr.b_conj_trans = 1;
-    if ((rc = launch_cgemm(gr, st))) return rc;
+    return rest(gr);
   }
+  // slice = (V D) H^H: n1 x n2 = q x p
+  CGemm gr{t.Gr, t.Gi, t.Hr, t.Hi, t.Mr, t.Mi, q, p, q, nullptr, q, p, q, q * q, p * q, q * p,
+           h, t.n3, TP_FP32, nullptr, nullptr, nullptr, nullptr, q, status};
+  gr.b_conj_trans = 1;
+  return rest(gr);
+}
+
+// One ADMM iteration of one tensor on stream st.
+int svt_iteration(const SvtTensor& t, bool warm, double rho, double mu_max, int sweeps,
+                  int32_t* status, cudaStream_t st) {
+  int rc;
+  const int64_t n = t.n1 * t.n2 * t.n3, n12 = t.n1 * t.n2;
+  {
+    KernelScope ks("admm_pre", st);
+    admm_pre_kernel<<<grid_n(n), 256, 0, st>>>(t.X, t.mask, t.E, t.Y, t.mu, n, t.M);
+  }
+  DftGather gm{t.M, n12, 1, 1, 0, n12, nullptr, nullptr, nullptr, 0, t.n3, t.Mr, t.Mi,
+               n12, n12, nullptr, nullptr, 0};
+  if ((rc = launch_rdft(gm, st))) return rc;
+  if ((rc = svt_shrink(t, warm, sweeps, status, st))) return rc;
   if ((rc = launch_irdft(t.Mr, t.Mi, n12, n12, t.n3, t.L, st))) return rc;
   {
     KernelScope ks("admm_post", st);
@@ -470,11 +608,13 @@ int svt_run(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int64_t
     return TP_EINVAL;
   }
   Arena ws;
-  int rc = acquire_workspace(opts, svt_ws(n1, n2, n3, prec), &ws);
+  const size_t need = svt_ws(n1, n2, n3, prec);
+  bool lean = false;   // without svt_top.cu's state every slice takes the Jacobi
+  int rc = acquire_workspace(opts, need, &ws, need - svt_top_bytes(n1, n2, n3), &lean);
   if (rc) return rc;
   int32_t* status = opts ? opts->status : nullptr;
   const int sweeps = (opts && opts->max_sweeps > 0) ? opts->max_sweeps : 30;
-  SvtTensor t = svt_carve(X, mask, n1, n2, n3, L, E, Y, mu, ws, prec);
+  SvtTensor t = svt_carve(X, mask, n1, n2, n3, L, E, Y, mu, ws, prec, lean);
   t.lam = lam;
   t.alone = true;
   if ((rc = svt_init(t, st))) return rc;
@@ -532,7 +672,11 @@ int svt_batched_run(int ntens, const tp_tensor_desc* d, int iters, double rho, d
     return TP_EINVAL;
   }
   Arena ws;
-  int rc = acquire_workspace(opts, svt_batched_ws(ntens, d, prec), &ws);
+  const size_t need = svt_batched_ws(ntens, d, prec);
+  size_t top = 0;
+  for (int i = 0; i < ntens; ++i) top += svt_top_bytes(d[i].n1, d[i].n2, d[i].n3);
+  bool lean = false;   // as in the single completion
+  int rc = acquire_workspace(opts, need, &ws, need - top, &lean);
   if (rc) return rc;
   if (iters <= 0) return TP_OK;
   int32_t* status = opts ? opts->status : nullptr;
@@ -541,7 +685,7 @@ int svt_batched_run(int ntens, const tp_tensor_desc* d, int iters, double rho, d
   T.reserve(size_t(ntens));
   for (int i = 0; i < ntens; ++i) {
     T.push_back(svt_carve(d[i].X, d[i].mask, d[i].n1, d[i].n2, d[i].n3, d[i].L, d[i].E, d[i].Y,
-                          d[i].mu, ws, prec));
+                          d[i].mu, ws, prec, lean));
     if (lams) T.back().lam = lams[i];   // > 0: robust form of problem tlow7
   }
   const int ns = ntens < kSideStreams ? ntens : kSideStreams;

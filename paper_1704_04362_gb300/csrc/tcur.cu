@@ -34,6 +34,7 @@ namespace tp {
 
 int launch_cgemm(const CGemm& g, cudaStream_t st);
 size_t svt_ws(int64_t n1, int64_t n2, int64_t n3, int prec = TP_FP32);
+size_t svt_top_bytes(int64_t n1, int64_t n2, int64_t n3);
 int svt_batched_run(int ntens, const tp_tensor_desc* d, int iters, double rho, double mu_max,
                     const tp_opts* opts, cudaStream_t st, const double* lams);
 int hybrid_svd(const float* xr, const float* xi, int64_t sX, int64_t ldx, bool conj, int p, int q,
@@ -543,7 +544,10 @@ int cur_tnn_run(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int
   const int64_t h = half_len(n3);
   const size_t N = size_t(n1) * n2 * n3;
   Arena ws;
-  int rc = acquire_workspace(opts, cur_tnn_ws(n1, n2, n3), &ws);
+  // a workspace without the completion's kept vectors does too (svt.cu)
+  const size_t need = cur_tnn_ws(n1, n2, n3), top = 2 * svt_top_bytes(n1, n2, n3);
+  bool lean = false;
+  int rc = acquire_workspace(opts, need, &ws, need - top, &lean);
   if (rc) return rc;
   int32_t* status = opts ? opts->status : nullptr;
   double* a2 = ws.take<double>(n2);
@@ -563,7 +567,8 @@ int cur_tnn_run(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int
   uint8_t* Rm = ws.take<uint8_t>(N);
   float* st_ws[6];
   for (int i = 0; i < 6; ++i) st_ws[i] = ws.take<float>(N);
-  char* admm_ws = ws.take<char>(2 * svt_ws(n1, n2, n3));
+  const size_t admm_bytes = 2 * svt_ws(n1, n2, n3) - (lean ? top : 0);
+  char* admm_ws = ws.take<char>(admm_bytes);
   float* Chr = ws.take<float>(size_t(n1) * n2 * h);
   float* Chi = ws.take<float>(size_t(n1) * n2 * h);
   float* Rhr = ws.take<float>(size_t(n1) * n2 * h);
@@ -669,7 +674,7 @@ int cur_tnn_run(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int
   tp_opts sub{};
   if (opts) sub = *opts;
   sub.workspace = admm_ws;
-  sub.workspace_bytes = 2 * svt_ws(n1, n2, n3);
+  sub.workspace_bytes = admm_bytes;
   if ((rc = svt_batched_run(2, d, iters, rho, mu_max, &sub, st, lams))) return rc;
   // 6-7. W~ = rows ridx of C~, L~ = C~ W~^dagger R~ per Fourier slice
   DftGather gc2{Ct, n1 * cp, 1, 1, 0, n1 * cp, nullptr, nullptr, nullptr, 0, n3, Chr, Chi,

@@ -118,6 +118,10 @@ struct CGemm {
   // FP32 path only: B_k(kk, n) = conj(b[k*sB + n + ldb*kk]) (B given as its
   // conjugate transpose)
   int b_conj_trans = 0;
+  // when non-null (device, one int per slice): only the slices f with
+  // only[f] == only_val are multiplied, the others' outputs stay as they are
+  const int* only = nullptr;
+  int only_val = 0;
   // tensor-core path: room for the partial sums of a K cut into parts
   // (cgemm_split_floats()), or null: K is not cut
   float* split_ws = nullptr;
