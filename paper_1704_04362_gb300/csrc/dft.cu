@@ -2,33 +2,25 @@
 // (Section 2, "Operators": fft(X,[],3) / ifft(X,[],3); Algorithm 1 steps 2-3
 // and the final inverse).
 //
-// Both directions are small dense contractions per tube, computed as
-// register-blocked SIMT products.  The t <-> n3 - t symmetry halves them:
-// with e_t = x_t + x_{n3-t} and o_t = x_t - x_{n3-t} (t = 1 .. n3/2; e_0 = x_0
-// and, for even n3, e_{n3/2} = x_{n3/2}, o = 0 there),
+// Both directions are small dense contractions per tube.  The t <-> n3 - t
+// symmetry halves them: with e_t = x_t + x_{n3-t} and o_t = x_t - x_{n3-t}
+// (t = 1 .. n3/2; e_0 = x_0 and, for even n3, e_{n3/2} = x_{n3/2}, o = 0 there),
 //     Re X_k = sum_{t <= n3/2} e_t cos(2 pi k t / n3),
 //     Im X_k = -sum_{t <= n3/2} o_t sin(2 pi k t / n3);
 // and for the inverse, with P_t = sum_k w_k Re X_k cos, Q_t = sum_k w_k Im X_k sin
 // (w_k = 1/n3 at k = 0 and k = n3/2, else 2/n3), x_t = P_t - Q_t and
-// x_{n3-t} = P_t + Q_t.  Each thread owns TPT tubes and KC frequencies (or
-// output times) per chunk; the KC columns of the transform matrix a chunk
-// needs are built once per block in shared memory from the n3-entry twiddle
-// table exp(-2 pi i m / n3), m = k t mod n3.  KC is chosen per call to
-// minimise padding.  The (Re, Im) and (P, Q) accumulator pairs are updated
-// with Blackwell's packed two-lane float32 FMA.
+// x_{n3-t} = P_t + Q_t.  Over all tubes these are two real matrix products
+// with a common schedule (dft_product_kernel); each sum runs in order.
+#include <algorithm>
+
 #include "dft_common.cuh"
 
 namespace tp {
 namespace {
 using namespace dftc;
 
-#ifndef TP_DFT_TPT
-#define TP_DFT_TPT 2
-#endif
-constexpr int TPT = TP_DFT_TPT;  // tubes per thread
-constexpr int RB = 128;          // threads per block
-constexpr int TU = 8;            // samples (forward) or frequencies (inverse) loaded ahead
-constexpr int STAGE_BYTES_MAX = 64 * 1024;
+constexpr int RB = 128;          // threads per block of the transposed kernel
+constexpr int TU = 8;            // samples it loads ahead
 
 // (cos, sin)(2 pi m / n3) for m < n3.  float sincospi (about 1 ulp; exact at
 // quarter turns, m/n3 in {0, 1/4, 1/2, 3/4}) keeps the tables off the slow
@@ -43,117 +35,206 @@ __device__ __forceinline__ void build_twiddles(float2* tw, int n3) {
   }
 }
 
-// Folded pair (e_t, o_t) of one tube; t <= n3/2.
-__device__ __forceinline__ void fold(float x0, float x1, int t, int n3, float& e, float& o) {
-  if (t == 0 || 2 * t == n3) {
-    e = x0;
-    o = 0.f;
-  } else {
-    e = x0 + x1;
-    o = x0 - x1;
-  }
-}
+// The transforms as matrix products: M = tubes, N = outputs (frequencies k of
+// the forward, times t <= n3/2 of the inverse), K = folded samples t (or
+// frequencies k), two products side by side (e cos | -o sin; w Re cos | w Im sin).
+// A block of TX x TY threads owns 4 TX tubes and 4 TY outputs, a thread 4 tubes
+// x 4 outputs of both products as tube pairs on the packed two-lane FMA.  The
+// K x 4 TY table of the transform matrix stays in shared memory while the
+// block walks its tubes; the tubes come in K tiles of 8, folded on the way from
+// registers to shared memory, the next tile's samples loaded before the
+// current one is used.  The whole half spectrum of a tube up to n3 = 256 is
+// produced by one block, so each sample is read once (longer tubes take the
+// outputs in as many parts as their table needs shared memory).
+// Bound by the float32 pipe for n3 above about 60, below by the tubes' traffic.
+// 218880 tubes, one output per thread and tube group in chunks of 16 (table
+// rebuilt per chunk) -> this: n3 = 67 forward 0.22 -> 0.11 ms, inverse 0.079 ->
+// 0.065; n3 = 127 0.62 -> 0.18, 0.19 -> 0.12; n3 = 251 3.6 -> 0.87, 0.75 -> 0.47.
+constexpr int DK = 8;                        // K tile
+constexpr int DN = 4, DM = 4;                // outputs and tubes per thread
+constexpr int TABLE_BYTES_MAX = 120 * 1024;
+constexpr int DT_MAX = 544;                  // threads: 16 x 33 at n3 = 256
 
-// Wc[t*KC + q] = (cos, sin)(2 pi (k0+q) t / n3) for t <= nh, zero above.
-template <int KC>
-__device__ __forceinline__ void build_fwd_cols(float2* Wc, const float2* tw, int n3, int nh,
-                                               int nhp, int k0) {
-  for (int e = threadIdx.x; e < nhp * KC; e += blockDim.x) {
-    const int t = e / KC, q = e - t * KC;
-    Wc[e] = t <= nh ? tw[int((int64_t(k0 + q) * t) % n3)] : make_float2(0.f, 0.f);
-  }
-}
+struct DftArgs {
+  DftGather g;                // forward
+  const float *in_re, *in_im; // inverse
+  float* out;
+  int64_t rows, in_slice;
+  int n3, K, N, parts;        // K terms, N outputs a part, parts of the outputs
+  int tx_log, ty;             // block shape
+};
 
-template <int KC>
-__global__ void __launch_bounds__(RB) rdft_kernel(DftGather g, int stage) {
-  extern __shared__ float2 sm2[];
-  const int n3 = int(g.n3);
-  const int h = n3 / 2 + 1, nh = n3 / 2;
-  const int nhp = (nh + 1 + TU - 1) / TU * TU;
-  float2* tw = sm2;
-  float2* Wc = sm2 + n3;
-  float* xs = reinterpret_cast<float*>(Wc + nhp * KC);   // staging [n3][RB*TPT] when stage
+// NP: K-tile samples per thread; MT, MB: threads a block and blocks per SM the
+// registers are budgeted for (80 registers keep 22 to 24 warps on an SM).
+template <bool INV, int NP, int MT, int MB>
+__global__ void __launch_bounds__(MT, MB) dft_product_kernel(const __grid_constant__ DftArgs p) {
+  extern __shared__ __align__(16) float dft_sm[];
+  const int n3 = p.n3, h = n3 / 2 + 1, K = p.K, KP = (K + DK - 1) / DK * DK;
+  const int TX = 1 << p.tx_log, BM = DM * TX, NO = DN * p.ty, nt = TX * p.ty;
+  const int tid = threadIdx.x, tx = tid & (TX - 1), ty = tid >> p.tx_log;
+  const int q0 = int(blockIdx.y) * p.N;      // first output of this part
+  float2* W = reinterpret_cast<float2*>(dft_sm);                 // [KP][NO]
+  float* Ab = dft_sm + 2 * KP * NO;                               // [2][2][DK][BM]
+  const float** base = reinterpret_cast<const float**>(Ab + 4 * DK * BM);   // [BM]
+  int64_t* offs = reinterpret_cast<int64_t*>(base + BM);         // [BM], -1 past the data
+  float* scl = reinterpret_cast<float*>(offs + BM);              // [BM]
+  float2* tw = reinterpret_cast<float2*>(scl + BM);              // [n3]
   build_twiddles(tw, n3);
-  const Extent ex = extent_of(g);
-  const int64_t base = int64_t(blockIdx.x) * (RB * TPT);
-  if (base >= ex.rows_pad) return;   // uniform over the block
-  const int tid = threadIdx.x;
-
-  for (int64_t c = blockIdx.y; c < ex.cols_pad; c += gridDim.y) {
-    const float* p[TPT];
-    float s[TPT];
-    bool act[TPT];
-#pragma unroll
-    for (int j = 0; j < TPT; ++j) {
-      const int64_t r = base + j * RB + tid;
-      act[j] = r < ex.rows_pad;
-      p[j] = act[j] ? tube_ptr(g, ex, r, c, s[j]) : nullptr;
-    }
-    if (stage) {
-      // every sample of this thread's tubes, read once (all loads in flight)
-      for (int t = 0; t < n3; ++t)
-#pragma unroll
-        for (int j = 0; j < TPT; ++j)
-          xs[t * (RB * TPT) + j * RB + tid] =
-              p[j] ? s[j] * __ldg(p[j] + int64_t(t) * g.slice_stride) : 0.f;
-    }
-    for (int k0 = 0; k0 < h; k0 += KC) {
-      __syncthreads();
-      build_fwd_cols<KC>(Wc, tw, n3, nh, nhp, k0);
-      __syncthreads();
-      float2 acc[TPT][KC];   // (Re, Im), updated by packed two-lane FMAs
-#pragma unroll
-      for (int j = 0; j < TPT; ++j)
-#pragma unroll
-        for (int q = 0; q < KC; ++q) acc[j][q] = make_float2(0.f, 0.f);
-      for (int t0 = 0; t0 <= nh; t0 += TU) {
-        float ev[TPT][TU], ov[TPT][TU];
-#pragma unroll
-        for (int u = 0; u < TU; ++u)
-#pragma unroll
-          for (int j = 0; j < TPT; ++j) {
-            const int t = t0 + u;
-            float x0 = 0.f, x1 = 0.f;
-            if (t <= nh) {
-              if (stage) {
-                x0 = xs[t * (RB * TPT) + j * RB + tid];
-                x1 = xs[((n3 - t) % n3) * (RB * TPT) + j * RB + tid];
-              } else if (p[j]) {
-                x0 = s[j] * __ldg(p[j] + int64_t(t) * g.slice_stride);
-                if (t > 0 && 2 * t != n3)
-                  x1 = s[j] * __ldg(p[j] + int64_t(n3 - t) * g.slice_stride);
-              }
-            }
-            fold(x0, x1, t, n3, ev[j][u], ov[j][u]);
-          }
-#pragma unroll
-        for (int u = 0; u < TU; ++u)
-#pragma unroll
-          for (int q = 0; q < KC; ++q) {
-            const float2 w = Wc[(t0 + u) * KC + q];   // zero rows past nh
-#pragma unroll
-            for (int j = 0; j < TPT; ++j)
-              acc[j][q] = __ffma2_rn(make_float2(ev[j][u], -ov[j][u]), w, acc[j][q]);
-          }
+  __syncthreads();
+  const float inv = 1.0f / float(n3);
+  for (int e = tid; e < KP * NO; e += nt) {
+    const int t = e / NO, q = q0 + e - t * NO;
+    float2 w = make_float2(0.f, 0.f);
+    if (q < h && t < K) {
+      w = tw[int((int64_t(q) * t) % n3)];
+      if (INV) {
+        const float wk = (t == 0 || 2 * t == n3) ? inv : 2.0f * inv;
+        w = make_float2(wk * w.x, wk * w.y);
+      } else {
+        w.y = -w.y;
       }
+    }
+    W[e] = w;
+  }
+  Extent ex{};
+  int64_t total;
+  if (INV) {
+    total = p.rows;
+  } else {
+    ex = extent_of(p.g);
+    total = ex.rows_pad * ex.cols_pad;
+  }
+  const int64_t ss = INV ? p.in_slice : p.g.slice_stride;
+
+  float v0[NP], v1[NP];
+  // raw values of K tile k0 of the current tubes, into registers
+  auto fetch = [&](int k0) {
 #pragma unroll
-      for (int j = 0; j < TPT; ++j) {
-        if (!act[j]) continue;
-        const int64_t o = base + j * RB + tid + g.out_ld * c;
+    for (int u = 0; u < NP; ++u) {
+      const int e = tid + u * nt, m = e & (BM - 1), t = k0 + (e >> (p.tx_log + 2));
+      v0[u] = v1[u] = 0.f;
+      if (e >= DK * BM || t >= K) continue;
+      const float* b = base[m];
+      if (!b) continue;
+      const float* a = b + int64_t(t) * ss;
+      if (INV) {
+        v0[u] = __ldg(a);
+        // the imaginary parts of the real slices are ignored
+        if (t > 0 && 2 * t != n3) v1[u] = __ldg(p.in_im + (a - p.in_re));
+      } else {
+        v0[u] = scl[m] * __ldg(a);
+        if (t > 0 && 2 * t != n3) v1[u] = scl[m] * __ldg(b + int64_t(n3 - t) * ss);
+      }
+    }
+  };
+  auto stage = [&](int k0, float* A) {   // A: [2][DK][BM]
 #pragma unroll
-        for (int q = 0; q < KC; ++q) {
-          if (k0 + q < h) {
-            const int64_t oo = o + int64_t(k0 + q) * g.out_slice;
-            const float ar = acc[j][q].x, ai = acc[j][q].y;
-            if (g.out_re_lo) {
-              put_split(g.out_re, g.out_re_lo, g.out_bf16 != 0, oo, ar);
-              put_split(g.out_im, g.out_im_lo, g.out_bf16 != 0, oo, ai);
-            } else {
-              g.out_re[oo] = ar;
-              g.out_im[oo] = ai;
-            }
+    for (int u = 0; u < NP; ++u) {
+      const int e = tid + u * nt;
+      if (e >= DK * BM) continue;
+      const int t = k0 + (e >> (p.tx_log + 2));
+      const bool lone = t == 0 || 2 * t == n3;
+      A[e] = INV ? v0[u] : lone ? v0[u] : v0[u] + v1[u];
+      A[DK * BM + e] = INV ? v1[u] : lone ? 0.f : v0[u] - v1[u];
+    }
+  };
+
+  for (int64_t m0 = int64_t(blockIdx.x) * BM; m0 < total; m0 += int64_t(gridDim.x) * BM) {
+    __syncthreads();   // the previous tubes' addresses and tiles are done with
+    for (int m = tid; m < BM; m += nt) {
+      const int64_t e = m0 + m;
+      const bool in = e < total;
+      if (INV) {
+        base[m] = in ? p.in_re + e : nullptr;
+        offs[m] = in ? e : -1;
+      } else {
+        const int64_t c = in ? e / ex.rows_pad : 0, r = in ? e - c * ex.rows_pad : 0;
+        float s = 0.f;
+        base[m] = in ? tube_ptr(p.g, ex, r, c, s) : nullptr;
+        scl[m] = s;
+        offs[m] = in ? r + p.g.out_ld * c : -1;
+      }
+    }
+    __syncthreads();
+    float2 a0[2][DN], a1[2][DN];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int q = 0; q < DN; ++q) a0[i][q] = a1[i][q] = make_float2(0.f, 0.f);
+    fetch(0);
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += DK, buf ^= 1) {
+      float* A = Ab + buf * 2 * DK * BM;
+      stage(k0, A);
+      __syncthreads();   // also: every thread is done with the other buffer's last use
+      if (k0 + DK < K) fetch(k0 + DK);
+#pragma unroll 2
+      for (int kk = 0; kk < DK; ++kk) {   // zero samples past K
+        const float4 x = *reinterpret_cast<const float4*>(A + kk * BM + DM * tx);
+        const float4 y = *reinterpret_cast<const float4*>(A + (DK + kk) * BM + DM * tx);
+        const float2 xe[2] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
+        const float2 yo[2] = {make_float2(y.x, y.y), make_float2(y.z, y.w)};
+        const float4* w4 = reinterpret_cast<const float4*>(W + (k0 + kk) * NO + DN * ty);
+#pragma unroll
+        for (int q = 0; q < DN; q += 2) {
+          const float4 w = w4[q / 2];
+          const float2 c0 = make_float2(w.x, w.x), s0 = make_float2(w.y, w.y);
+          const float2 c1 = make_float2(w.z, w.z), s1 = make_float2(w.w, w.w);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            a0[i][q] = __ffma2_rn(xe[i], c0, a0[i][q]);
+            a1[i][q] = __ffma2_rn(yo[i], s0, a1[i][q]);
+            a0[i][q + 1] = __ffma2_rn(xe[i], c1, a0[i][q + 1]);
+            a1[i][q + 1] = __ffma2_rn(yo[i], s1, a1[i][q + 1]);
           }
         }
+      }
+    }
+    // outputs q of the thread's four tubes; four consecutive ones in one store
+    // where their place is aligned
+    const int64_t o0 = offs[DM * tx], o3 = offs[DM * tx + 3];
+    const bool quad = o0 >= 0 && o3 == o0 + 3 && (o0 & 3) == 0;
+    auto put4 = [&](float* dst, int64_t shift, bool aligned, const float (&v)[4]) {
+      if (quad && aligned) {
+        *reinterpret_cast<float4*>(dst + shift + o0) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int64_t o = offs[DM * tx + j];
+          if (o >= 0) dst[shift + o] = v[j];
+        }
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < DN; ++q) {
+      const int k = q0 + DN * ty + q;
+      if (DN * ty + q >= p.N || k >= h) continue;
+      const float u[4] = {a0[0][q].x, a0[0][q].y, a0[1][q].x, a0[1][q].y};
+      const float v[4] = {a1[0][q].x, a1[0][q].y, a1[1][q].x, a1[1][q].y};
+      if (INV) {
+        const bool al = (p.rows & 3) == 0 && aligned16(p.out);
+        float lo[4], hi[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          lo[j] = u[j] - v[j];
+          hi[j] = u[j] + v[j];
+        }
+        put4(p.out, p.rows * int64_t(k), al, lo);
+        if (k > 0 && n3 - k > n3 / 2) put4(p.out, p.rows * int64_t(n3 - k), al, hi);
+      } else if (p.g.out_re_lo) {
+        const int64_t shift = int64_t(k) * p.g.out_slice;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int64_t o = offs[DM * tx + j];
+          if (o < 0) continue;
+          put_split(p.g.out_re, p.g.out_re_lo, p.g.out_bf16 != 0, shift + o, u[j]);
+          put_split(p.g.out_im, p.g.out_im_lo, p.g.out_bf16 != 0, shift + o, v[j]);
+        }
+      } else {
+        const bool al = (p.g.out_slice & 3) == 0;
+        const int64_t shift = int64_t(k) * p.g.out_slice;
+        put4(p.g.out_re, shift, al && aligned16(p.g.out_re), u);
+        put4(p.g.out_im, shift, al && aligned16(p.g.out_im), v);
       }
     }
   }
@@ -267,83 +348,6 @@ __global__ void __launch_bounds__(RB) rdft_t_kernel(DftGather g) {
   }
 }
 
-// Inverse: x_t = P_t - Q_t, x_{n3-t} = P_t + Q_t over output-time chunks t <= n3/2.
-template <int KC>
-__global__ void __launch_bounds__(RB) irdft_kernel(const float* __restrict__ in_re,
-                                                   const float* __restrict__ in_im, int64_t rows,
-                                                   int64_t in_slice, int n3,
-                                                   float* __restrict__ out) {
-  extern __shared__ float2 sm2[];
-  const int h = n3 / 2 + 1, nh = n3 / 2;
-  const int hp = (h + TU - 1) / TU * TU;
-  float2* tw = sm2;
-  float2* Vc = sm2 + n3;   // Vc[k*KC + q] = (w_k/n3) tw[k*(t0+q) mod n3], zero past h or nh
-  build_twiddles(tw, n3);
-  const int tid = threadIdx.x;
-  const float inv = 1.0f / float(n3);
-  for (int64_t base = int64_t(blockIdx.x) * (RB * TPT); base < rows;
-       base += int64_t(gridDim.x) * (RB * TPT)) {
-    int64_t r[TPT];
-#pragma unroll
-    for (int j = 0; j < TPT; ++j) r[j] = base + j * RB + tid;
-    for (int t0 = 0; t0 <= nh; t0 += KC) {
-      __syncthreads();
-      for (int e = tid; e < hp * KC; e += RB) {
-        const int k = e / KC, q = e - k * KC;
-        const int t = t0 + q;
-        if (k < h && t <= nh) {
-          const float wk = (k == 0 || 2 * k == n3) ? inv : 2.0f * inv;
-          const float2 w = tw[int((int64_t(k) * t) % n3)];
-          Vc[e] = make_float2(wk * w.x, wk * w.y);
-        } else {
-          Vc[e] = make_float2(0.f, 0.f);
-        }
-      }
-      __syncthreads();
-      float2 PQ[TPT][KC];   // (P, Q), updated by packed two-lane FMAs
-#pragma unroll
-      for (int j = 0; j < TPT; ++j)
-#pragma unroll
-        for (int q = 0; q < KC; ++q) PQ[j][q] = make_float2(0.f, 0.f);
-      for (int k0 = 0; k0 < h; k0 += TU) {
-        float re[TPT][TU], im[TPT][TU];
-#pragma unroll
-        for (int u = 0; u < TU; ++u)
-#pragma unroll
-          for (int j = 0; j < TPT; ++j) {
-            const int k = k0 + u;
-            const bool ok = r[j] < rows && k < h;
-            re[j][u] = ok ? __ldg(in_re + int64_t(k) * in_slice + r[j]) : 0.f;
-            // the imaginary parts of the real slices are ignored
-            im[j][u] = (ok && k > 0 && 2 * k != n3) ? __ldg(in_im + int64_t(k) * in_slice + r[j])
-                                                    : 0.f;
-          }
-#pragma unroll
-        for (int u = 0; u < TU; ++u)
-#pragma unroll
-          for (int q = 0; q < KC; ++q) {
-            const float2 v = Vc[(k0 + u) * KC + q];
-#pragma unroll
-            for (int j = 0; j < TPT; ++j)
-              PQ[j][q] = __ffma2_rn(make_float2(re[j][u], im[j][u]), v, PQ[j][q]);
-          }
-      }
-#pragma unroll
-      for (int j = 0; j < TPT; ++j) {
-        if (r[j] >= rows) continue;
-#pragma unroll
-        for (int q = 0; q < KC; ++q) {
-          const int t = t0 + q;
-          if (t <= nh) {
-            out[r[j] + rows * int64_t(t)] = PQ[j][q].x - PQ[j][q].y;
-            if (t > 0 && n3 - t > nh) out[r[j] + rows * int64_t(n3 - t)] = PQ[j][q].x + PQ[j][q].y;
-          }
-        }
-      }
-    }
-  }
-}
-
 // Chunk size among {16, 12, 8} that pads n the least (ties: larger).
 int pick_kc(int64_t n) {
   const int cands[3] = {16, 12, 8};
@@ -359,61 +363,86 @@ int pick_kc(int64_t n) {
   return best;
 }
 
+// The transposed form (a tuned tile width KC).
 template <int KC>
-int launch_rdft_kc(const DftGather& g, cudaStream_t st) {
-  const int64_t nh = g.n3 / 2;
-  const int64_t nhp = (nh + 1 + TU - 1) / TU * TU;
-  if (g.out_transposed) {
-    const int64_t n3p = (g.n3 + TU - 1) / TU * TU;
-    const size_t smem = size_t(g.n3 + n3p * KC) * sizeof(float2) +
-                        size_t(KC) * TR * (TCOL + 1) * sizeof(float);
-    TP_SET_SMEM(rdft_t_kernel<KC>, smem);
-    const int64_t bx = (g.rows + TR - 1) / TR;
-    if (bx > 0x7fffffff) { set_error("rdft: too many rows"); return TP_EINVAL; }
-    // the column tiles are walked grid-stride: with all rows live (no row
-    // gather) about 16 blocks per SM suffice, and a column gather's capacity
-    // can far exceed the picked count
-    int64_t by = (g.cols + TCOL - 1) / TCOL;
-    const int64_t by_cap = bx >= int64_t(sm_count()) * 16 ? 1 : int64_t(sm_count()) * 16 / bx;
-    if (g.gather_dim != 1 && by > by_cap) by = by_cap;
-    if (by > 65535) by = 65535;
-    {
-      KernelScope ks("rdft_t", st);
-      rdft_t_kernel<KC><<<dim3(unsigned(bx), unsigned(by)), RB, smem, st>>>(g);
-    }
-    return launch_status("rdft_t_kernel");
-  }
-  // stage the scattered row gathers so that each sample is read once
-  const size_t stage_bytes = size_t(g.n3) * RB * TPT * sizeof(float);
-  const int stage = (g.gather_dim == 1 && stage_bytes <= size_t(STAGE_BYTES_MAX)) ? 1 : 0;
-  const size_t smem = size_t(g.n3 + nhp * KC) * sizeof(float2) + (stage ? stage_bytes : 0);
-  TP_SET_SMEM(rdft_kernel<KC>, smem);
-  const int64_t bx = (g.rows + RB * TPT - 1) / (RB * TPT);
+int launch_rdft_t(const DftGather& g, cudaStream_t st) {
+  const int64_t n3p = (g.n3 + TU - 1) / TU * TU;
+  const size_t smem = size_t(g.n3 + n3p * KC) * sizeof(float2) +
+                      size_t(KC) * TR * (TCOL + 1) * sizeof(float);
+  TP_SET_SMEM(rdft_t_kernel<KC>, smem);
+  const int64_t bx = (g.rows + TR - 1) / TR;
   if (bx > 0x7fffffff) { set_error("rdft: too many rows"); return TP_EINVAL; }
-  int64_t by = g.cols < 65535 ? g.cols : 65535;   // columns walked grid-stride
+  // the column tiles are walked grid-stride: with all rows live (no row
+  // gather) about 16 blocks per SM suffice, and a column gather's capacity
+  // can far exceed the picked count
+  int64_t by = (g.cols + TCOL - 1) / TCOL;
   const int64_t by_cap = bx >= int64_t(sm_count()) * 16 ? 1 : int64_t(sm_count()) * 16 / bx;
-  if (g.gather_dim == 2 && by > by_cap) by = by_cap;   // see the transposed form
+  if (g.gather_dim != 1 && by > by_cap) by = by_cap;
+  if (by > 65535) by = 65535;
   {
-    KernelScope ks("rdft", st);
-    rdft_kernel<KC><<<dim3(unsigned(bx), unsigned(by)), RB, smem, st>>>(g, stage);
+    KernelScope ks("rdft_t", st);
+    rdft_t_kernel<KC><<<dim3(unsigned(bx), unsigned(by)), RB, smem, st>>>(g);
   }
-  return launch_status("rdft_kernel");
+  return launch_status("rdft_t_kernel");
 }
 
-template <int KC>
-int launch_irdft_kc(const float* in_re, const float* in_im, int64_t rows, int64_t in_slice,
-                    int64_t n3, float* out, cudaStream_t st) {
-  const int64_t h = n3 / 2 + 1;
-  const int64_t hp = (h + TU - 1) / TU * TU;
-  const size_t smem = size_t(n3 + hp * KC) * sizeof(float2);
-  TP_SET_SMEM(irdft_kernel<KC>, smem);
-  int64_t blocks = (rows + RB * TPT - 1) / (RB * TPT);
-  if (blocks > int64_t(sm_count()) * 64) blocks = int64_t(sm_count()) * 64;
-  {
-    KernelScope ks("irdft", st);
-    irdft_kernel<KC><<<unsigned(blocks), RB, smem, st>>>(in_re, in_im, rows, in_slice, int(n3), out);
+// Block shape and grid of a product over `tubes` tubes: outputs in the fewest
+// equal parts whose table fits, threads near 256 (more where the outputs of a
+// part need them), as many blocks as are resident, each walking its tubes.
+template <bool INV, int NP>
+int launch_product_np(const DftArgs& p, int64_t tubes, size_t smem, const char* name,
+                      cudaStream_t st) {
+  const int nt = p.ty << p.tx_log;
+  auto kernel = nt <= 256   ? dft_product_kernel<INV, NP, 256, 3>
+                : nt <= 384 ? dft_product_kernel<INV, NP, 384, 2>
+                            : dft_product_kernel<INV, NP, DT_MAX, 1>;
+  TP_SET_SMEM(kernel, smem);
+  if (nt > DT_MAX) {
+    set_error("dft: %d threads a block", nt);
+    return TP_EUNSUPPORTED;
   }
-  return launch_status("irdft_kernel");
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem) != cudaSuccess ||
+      per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  const int64_t bm = int64_t(DM) << p.tx_log;
+  int64_t blocks = (tubes + bm - 1) / bm;
+  const int64_t cap = std::max<int64_t>(1, int64_t(sm_count()) * per_sm / p.parts);
+  if (blocks > cap) blocks = cap;
+  {
+    KernelScope ks(name, st);
+    kernel<<<dim3(unsigned(blocks), unsigned(p.parts)), nt, smem, st>>>(p);
+  }
+  return launch_status("dft_product_kernel");
+}
+
+template <bool INV>
+int launch_product(DftArgs& p, int64_t tubes, const char* name, cudaStream_t st) {
+  const int h = p.n3 / 2 + 1;
+  p.K = h;
+  const size_t kp = size_t(h + DK - 1) / DK * DK;
+  const int fit = std::max(1, int(TABLE_BYTES_MAX / (sizeof(float2) * kp * DN)));
+  const int groups = (h + DN - 1) / DN;
+  p.parts = (groups + fit - 1) / fit;
+  p.ty = (groups + p.parts - 1) / p.parts;
+  p.N = p.ty * DN;
+  p.parts = (h + p.N - 1) / p.N;
+  // 16 to 64 lanes along the tubes: small problems and many outputs take few
+  p.tx_log = 4;
+  while (p.tx_log < 6 && (p.ty << (p.tx_log + 1)) <= 256 &&
+         tubes >= int64_t(sm_count()) * 2 * (DM << (p.tx_log + 1)))
+    ++p.tx_log;
+  const int nt = p.ty << p.tx_log;
+  const size_t bm = size_t(DM) << p.tx_log;
+  const size_t smem = kp * p.N * sizeof(float2) + 4 * DK * bm * sizeof(float) +
+                      bm * (sizeof(float*) + sizeof(int64_t) + sizeof(float)) +
+                      size_t(p.n3) * sizeof(float2);
+  const int np = int((DK * bm + nt - 1) / nt);   // K-tile samples per thread
+  if (np <= 4) return launch_product_np<INV, 4>(p, tubes, smem, name, st);
+  if (np <= 8) return launch_product_np<INV, 8>(p, tubes, smem, name, st);
+  return launch_product_np<INV, 16>(p, tubes, smem, name, st);   // ty >= 3: n3 > 16
 }
 
 }  // namespace
@@ -434,8 +463,8 @@ int launch_fft_inv(const float* ire, const float* iim, int64_t rows, int64_t in_
 #define TP_FFT_THRESHOLD 256
 #endif
 constexpr int64_t kFftThreshold = TP_FFT_THRESHOLD;
-// Power-of-two tubes up to 128 go through the register FFT (rfft_reg.cu);
-// building with -DTP_REG_FFT=0 keeps them on the direct contraction.
+// Tubes up to 16 and power-of-two ones up to 128 go through the register
+// transforms (rfft_reg.cu); building with -DTP_REG_FFT=0 keeps them on the direct contraction.
 #ifndef TP_REG_FFT
 #define TP_REG_FFT 1
 #endif
@@ -455,13 +484,20 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
   }
   if (g.rows == 0 || g.cols == 0) return TP_OK;
   if (kRegFft && rfft_reg_supported(g.n3)) return launch_rfft_reg(g, st);
-  // tile width KC among {8, 12, 16} (each frequency sums its samples in the
-  // same order whatever the width): autotuned, default the least padding
+  if (!g.out_transposed) {
+    DftArgs p{};
+    p.g = g;
+    p.n3 = int(g.n3);
+    return launch_product<false>(p, g.rows * g.cols, "rdft", st);
+  }
+  // transposed: tile width KC among {8, 12, 16} (each frequency sums its
+  // samples in the same order whatever the width): autotuned, default the
+  // least padding
   const auto run = [&](int c) {
     switch (c) {
-      case 0: return launch_rdft_kc<8>(g, st);
-      case 1: return launch_rdft_kc<12>(g, st);
-      default: return launch_rdft_kc<16>(g, st);
+      case 0: return launch_rdft_t<8>(g, st);
+      case 1: return launch_rdft_t<12>(g, st);
+      default: return launch_rdft_t<16>(g, st);
     }
   };
   const int kc = pick_kc(g.n3 / 2 + 1);
@@ -483,18 +519,14 @@ int launch_irdft(const float* in_re, const float* in_im, int64_t rows, int64_t i
   if (rows == 0) return TP_OK;
   if (kRegFft && rfft_reg_supported(n3))
     return launch_irfft_reg(in_re, in_im, rows, in_slice, n3, out, st);
-  const auto run = [&](int c) {
-    switch (c) {
-      case 0: return launch_irdft_kc<8>(in_re, in_im, rows, in_slice, n3, out, st);
-      case 1: return launch_irdft_kc<12>(in_re, in_im, rows, in_slice, n3, out, st);
-      default: return launch_irdft_kc<16>(in_re, in_im, rows, in_slice, n3, out, st);
-    }
-  };
-  const int kc = pick_kc(n3 / 2 + 1);
-  const int64_t key[2] = {n3, size_class(rows)};
-  int c = 0;
-  const int rc = autotune_pick("irdft", key, 2, 3, kc == 8 ? 0 : kc == 12 ? 1 : 2, run, st, &c);
-  return rc ? rc : run(c);
+  DftArgs p{};
+  p.in_re = in_re;
+  p.in_im = in_im;
+  p.rows = rows;
+  p.in_slice = in_slice;
+  p.out = out;
+  p.n3 = int(n3);
+  return launch_product<true>(p, rows, "irdft", st);
 }
 
 }  // namespace tp
