@@ -241,6 +241,7 @@ struct HqrParams {
   const int* ex_in;        // exponents of this level's source blocks (lfull rows each) or null
   int* flag;               // [slice]: 0, 1 (zero), 2 (not finite)
   int32_t* status;
+  int* weak;               // see householder.cuh
 };
 
 __device__ __forceinline__ void hqr_block(int rows, int nb, int b, int& r0, int& p) {
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(32 * W, HqrResident<R2, W, SLOTS>::v)
   constexpr int PP = 32 * R2;                          // row pairs of a column
   extern __shared__ __align__(16) float4 hqr_v[];      // reflectors, l columns of PP pairs
   __shared__ float2 tau_s[HQR_MAX_L];
-  __shared__ float sgn_s[HQR_MAX_L];                   // sign of R(j, j)
+  __shared__ float beta_s[HQR_MAX_L];                  // R(j, j)
   __shared__ int amax_s, bits_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int f = int(blockIdx.x) / g.nb, b = int(blockIdx.x) - f * g.nb;
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(32 * W, HqrResident<R2, W, SLOTS>::v)
         const float2 t = hqr_reflector<R2>(x[s0], kn, hqr_v + kn * PP, lane, beta);
         if (lane == 0) {
           tau_s[kn] = t;
-          sgn_s[kn] = beta < 0.f ? -1.f : 1.f;
+          beta_s[kn] = beta;
         }
       }
       if (live) hqr_apply<R2, W, SLOTS>(v, x, s0, kn, l, fc, warp, lane);
@@ -411,6 +412,24 @@ __global__ void __launch_bounds__(32 * W, HqrResident<R2, W, SLOTS>::v)
       if (bad && g.status) atomicOr(g.status, TP_DEV_BREAKDOWN);
     }
   }
+  if (g.weak && warp == 0) {
+    float lo = INFINITY, hi = 0.f;
+    bool nan = false;
+    for (int j = lane; j < l; j += 32) {
+      const float a = fabsf(beta_s[j]);
+      nan |= isnan(a);
+      lo = fminf(lo, a);
+      hi = fmaxf(hi, a);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    nan = __any_sync(0xffffffffu, nan);
+    const bool sound = !nan && lo > HQR_WEAK * hi && hi > 0x1p-40f && hi < 0x1p40f;
+    if (lane == 0 && !sound) atomicOr(g.weak, 1);
+  }
   // Q's column k: H_k e_k = e_k - tau_k v_k, then H_{k-1}, ..., H_0
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s) {
@@ -438,7 +457,7 @@ __global__ void __launch_bounds__(32 * W, HqrResident<R2, W, SLOTS>::v)
   for (int s = 0; s < SLOTS; ++s) {
     const int k = warp + W * s;
     if (k >= lfull) continue;
-    const float sg = (g.keep_phase && k < l) ? sgn_s[k] : 1.f;
+    const float sg = (g.keep_phase && k < l && beta_s[k] < 0.f) ? -1.f : 1.f;
 #pragma unroll
     for (int i = 0; i < 2 * R2; ++i) {
       const int r = 64 * (i >> 1) + 2 * lane + (i & 1);
@@ -568,7 +587,7 @@ constexpr int HQR_BLOCK = 256;
 bool householder_applies(int64_t p, int64_t l) { return p <= HQR_BLOCK && l <= HQR_MAX_L; }
 
 int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
-                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp) {
+                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp, int* weak) {
   if (p > HQR_BLOCK || l > HQR_MAX_L || l > p) {
     set_error("householder: needs l <= p <= %d and l <= %d", HQR_BLOCK, HQR_MAX_L);
     return TP_EUNSUPPORTED;
@@ -584,6 +603,7 @@ int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int
   g.lcols = lcols;
   g.keep_phase = keep_phase ? 1 : 0;
   g.sp = sp;
+  g.weak = weak;
   return hqr_dispatch<HQR_WHOLE>(g, p, batch, st);
 }
 
@@ -601,7 +621,8 @@ size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch) {
 }
 
 int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
-                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st) {
+                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st,
+                            int* weak) {
   constexpr int kMaxLevels = 24;   // each level shrinks the rows by 256 / 96 at least
   if (l < 1 || l > HQR_MAX_L || rows <= HQR_BLOCK || rows > 0x7fffffff) {
     set_error("householder_tall: needs more than %d rows and l <= %d", HQR_BLOCK, HQR_MAX_L);
@@ -627,6 +648,7 @@ int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int
     g.ex_in = ex;
     g.flag = flag;
     g.status = status;
+    g.weak = weak;
     if (batch * g.nb > 0x7fffffff || (g.nb > 1 && n == kMaxLevels)) {
       set_error("householder_tall: too many blocks");
       return TP_EUNSUPPORTED;

@@ -7,6 +7,12 @@ namespace tp {
 
 constexpr int HQR_MAX_L = 96;   // columns of a slice
 
+// weak (device, or null) of the launches below is set to 1 if some slice's
+// diagonal of R leaves the rank in doubt: min |R(j, j)| <= HQR_WEAK max
+// |R(j, j)|, or a maximum outside 2^-40 .. 2^40 (where float32 squares stop
+// being safe) or not finite.  2^-16 is 256 times float32's rounding.
+constexpr float HQR_WEAK = 1.f / 65536.f;
+
 // Split planes (p0 non-null): Q also leaves as the hi/lo planes (bf16 or
 // tf32, dftc::put_split) of the next tensor-core product's B operand,
 // K-major with leading dimension ldk, p <= ldk <= 32 ceil(p / 32) (rows
@@ -31,7 +37,8 @@ bool householder_applies(int64_t p, int64_t l);
 // nearly orthonormal columns Q(:, j) stays close to Y(:, j) instead of
 // possibly flipping its sign.
 int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
-                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{});
+                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{},
+                       int* weak = nullptr);
 
 // The same for contiguous slices of more than 256 rows (slice stride rows * l),
 // with `scratch` of householder_tall_scratch() bytes, 256-byte aligned.  A
@@ -39,6 +46,7 @@ int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int
 // (not a number).
 size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch);
 int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
-                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st);
+                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st,
+                            int* weak = nullptr);
 
 }  // namespace tp
