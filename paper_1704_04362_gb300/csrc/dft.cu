@@ -452,15 +452,18 @@ bool rfft_reg_supported(int64_t n3);
 int launch_rfft_reg(const DftGather& g, cudaStream_t st);
 int launch_irfft_reg(const float* in_re, const float* in_im, int64_t rows, int64_t in_slice,
                      int64_t n3, float* out, cudaStream_t st);
-int launch_fft_fwd(const float* X, int64_t rows, int64_t n3, float* ore, float* oim,
-                   int64_t out_slice, cudaStream_t st);
+int launch_fft_fwd(const DftGather& g, cudaStream_t st);
 int launch_fft_inv(const float* ire, const float* iim, int64_t rows, int64_t in_slice, int64_t n3,
                    float* out, cudaStream_t st);
 
-// Tubes longer than this go through the shared-memory FFT when their length
-// factors into small radices and no gather or split output is asked for.
+// Longer tubes than this go through the mixed-radix FFT (fft.cu) when their
+// length factors into primes up to 13; building with another value keeps
+// shorter ones on the direct contraction.  218880 tubes, FFT against product,
+// forward / inverse in us: n3 = 80 57 / 53 against 123 / 84; n3 = 225 (odd: a
+// full complex transform) 183 / 247 against 657 / 419; n3 = 45 on 237679 tubes
+// and less 27 / 47 against 45 / 46; level below.
 #ifndef TP_FFT_THRESHOLD
-#define TP_FFT_THRESHOLD 256
+#define TP_FFT_THRESHOLD 16
 #endif
 constexpr int64_t kFftThreshold = TP_FFT_THRESHOLD;
 // Tubes up to 16 and power-of-two ones up to 128 go through the register
@@ -475,15 +478,14 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
                      (g.cols == 1 || g.col_stride == g.rows) && g.out_ld == g.rows &&
                      g.out_slice == g.rows * g.cols && g.slice_stride == g.rows * g.cols &&
                      g.row_stride == 1;
-  if (plain && g.n3 > kFftThreshold && fft_supported(g.n3))
-    return launch_fft_fwd(g.src, g.rows * g.cols, g.n3, g.out_re, g.out_im, g.out_slice, st);
-  if (g.n3 < 1 || g.n3 > 512) {
+  if (g.n3 < 1 || (g.n3 > 512 && !(plain && fft_supported(g.n3)))) {
     set_error("rdft: n3 = %lld: longer than 512 needs a plain (ungathered) transform and "
               "prime factors <= 13", (long long)g.n3);
     return TP_EUNSUPPORTED;
   }
   if (g.rows == 0 || g.cols == 0) return TP_OK;
   if (kRegFft && rfft_reg_supported(g.n3)) return launch_rfft_reg(g, st);
+  if (g.n3 > kFftThreshold && fft_supported(g.n3)) return launch_fft_fwd(g, st);
   if (!g.out_transposed) {
     DftArgs p{};
     p.g = g;
@@ -510,15 +512,15 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
 
 int launch_irdft(const float* in_re, const float* in_im, int64_t rows, int64_t in_slice,
                  int64_t n3, float* out, cudaStream_t st) {
-  if (n3 > kFftThreshold && fft_supported(n3))
-    return launch_fft_inv(in_re, in_im, rows, in_slice, n3, out, st);
-  if (n3 < 1 || n3 > 512) {
+  if (n3 < 1 || (n3 > 512 && !fft_supported(n3))) {
     set_error("irdft: n3 = %lld: longer than 512 needs prime factors <= 13", (long long)n3);
     return TP_EUNSUPPORTED;
   }
   if (rows == 0) return TP_OK;
   if (kRegFft && rfft_reg_supported(n3))
     return launch_irfft_reg(in_re, in_im, rows, in_slice, n3, out, st);
+  if (n3 > kFftThreshold && fft_supported(n3))
+    return launch_fft_inv(in_re, in_im, rows, in_slice, n3, out, st);
   DftArgs p{};
   p.in_re = in_re;
   p.in_im = in_im;
