@@ -7,6 +7,9 @@ namespace tp {
 
 int launch_cgemm_simt(const CGemm& g, cudaStream_t st);
 int launch_cgemm_tc(const CGemm& g, cudaStream_t st);
+bool tprod_small_applies(int64_t n1, int64_t n2, int64_t n4, int64_t n3);
+int launch_tprod_small(const float* A, const float* B, float* C, int64_t n1, int64_t n2,
+                       int64_t n4, int64_t n3, cudaStream_t st);
 
 int launch_cgemm(const CGemm& g, cudaStream_t st) {
   if (g.precision == TP_FP32) return launch_cgemm_simt(g, st);
@@ -60,15 +63,23 @@ Planes take_planes(Arena& ws, size_t elems, bool tc) {
   return p;
 }
 
+// Whether the two arrays share no element (the one-launch product reads its
+// operands while it writes C; the general one has read them by then).
+bool apart(const float* x, int64_t nx, const float* y, int64_t ny) {
+  const auto a = reinterpret_cast<uintptr_t>(x), b = reinterpret_cast<uintptr_t>(y);
+  return a + uintptr_t(nx) * sizeof(float) <= b || b + uintptr_t(ny) * sizeof(float) <= a;
+}
+
+// Room for the K parts' sums of the product (0: K stays whole).
+size_t split_bytes(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
+  return is_tc(prec) ? ws_bytes(cgemm_split_floats(n1, n4, half_len(n3), n2, prec), 4) : 0;
+}
+
 // Operand layouts.  SIMT: A_hat_k is n1 x K column-major (leading dimension
 // n1).  Tensor cores: A_hat_k is stored K-major, element (i, kk) at
 // kk + lk*i with lk = K padded to 16 bytes (4 floats for 3xTF32, 8 bf16 for
 // BF16x3).  B_hat_k is K-major in both (leading dimension K, padded likewise
 // for the tensor cores).  The planes are sized as floats in both splits.
-size_t split_bytes(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
-  return is_tc(prec) ? ws_bytes(cgemm_split_floats(n1, n4, half_len(n3), n2, prec), 4) : 0;
-}
-
 size_t tprod_ws(int64_t n1, int64_t n2, int64_t n4, int64_t n3, int prec) {
   const size_t h = size_t(half_len(n3));
   const bool tc = is_tc(prec);
@@ -119,6 +130,9 @@ int tprod(const float* A, const float* B, float* C, int64_t n1, int64_t n2, int6
   bool lean = false;
   int rc = acquire_workspace(opts, need, &ws, need - split, &lean);
   if (rc) return rc;
+  if (!tc && tprod_small_applies(n1, n2, n4, n3) && apart(C, n1 * n4 * n3, A, n1 * n2 * n3) &&
+      apart(C, n1 * n4 * n3, B, n2 * n4 * n3))
+    return launch_tprod_small(A, B, C, n1, n2, n4, n3, st);
   const int64_t h = half_len(n3);
   const int64_t lk = pad_k(n2, prec);              // K leading dimension
   const int64_t la = tc ? lk : n1;                 // A leading dimension
