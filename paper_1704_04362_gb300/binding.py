@@ -241,11 +241,21 @@ def _check(rc: int, what: str):
 
 # ---------------------------------------------------------------- torch plumbing
 
+# The argument handling below runs several times per call and was 31 of the 49
+# us of a 64 x 48 x 32 x 16 product (device queries, stream objects, a permuted
+# allocation): the module is looked up once, the raw stream handle is asked for
+# without building a Stream, and layouts are compared by their strides.
+_TORCH = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise TprodError("libtprod needs a CUDA device; there is no CPU path")
-    return torch
+    global _TORCH
+    if _TORCH is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise TprodError("libtprod needs a CUDA device; there is no CPU path")
+        _TORCH = torch
+    return _TORCH
 
 
 def empty_tensor(n1, n2, n3, dtype=None, device=None):
@@ -253,7 +263,7 @@ def empty_tensor(n1, n2, n3, dtype=None, device=None):
     torch = _torch()
     dtype = dtype or torch.float32
     device = device or torch.device("cuda", torch.cuda.current_device())
-    return torch.empty((n3, n2, n1), dtype=dtype, device=device).permute(2, 1, 0)
+    return torch.empty_strided((n1, n2, n3), (1, n1, n1 * n2), dtype=dtype, device=device)
 
 
 def as_tprod_layout(x, dtype=None):
@@ -286,16 +296,18 @@ def _tensor_arg(x, name, dtype=None):
         raise TprodError(f"{name} must be a CUDA torch tensor")
     if x.dtype != dtype:
         raise TprodError(f"{name} must be {dtype}, got {x.dtype}")
-    if x.dim() == 3 and not _is_colmajor(x):
-        raise TprodError(f"{name} must be column-major (use as_tprod_layout)")
-    if x.dim() != 3 and not x.is_contiguous():
+    if x.dim() == 3:
+        n1, n2, _ = x.shape
+        if x.stride() != (1, n1, n1 * n2) and not _is_colmajor(x):
+            raise TprodError(f"{name} must be column-major (use as_tprod_layout)")
+    elif not x.is_contiguous():
         raise TprodError(f"{name} must be contiguous")
-    return ctypes.c_void_p(x.data_ptr())
+    return x.data_ptr()
 
 
 def _stream():
     torch = _torch()
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 _WS = {}
@@ -307,7 +319,7 @@ def _opts(op, dims, precision=TP_FP32, status=None, max_sweeps=0, wait_limit=0):
     L = lib()
     d = (ctypes.c_int64 * len(dims))(*[int(v) for v in dims])
     o = TpOpts(int(precision), int(max_sweeps), None, 0, None, int(wait_limit))
-    need = int(L.tp_workspace_query(op, ctypes.cast(d, ctypes.c_void_p), len(dims), ctypes.byref(o)))
+    need = L.tp_workspace_query(op, ctypes.addressof(d), len(dims), ctypes.byref(o))
     dev = torch.cuda.current_device()
     buf = _WS.get(dev)
     if need > 0 and (buf is None or buf.numel() < need):
@@ -470,11 +482,9 @@ def tcomplete_svt_batched(tensors, iters, rho=1.1, mu_max=1e10, status=None, max
     dims = []
     for i, (X, mask, L, E, Y, mu) in enumerate(tensors):
         n1, n2, n3 = X.shape
-        descs[i] = TpTensorDesc(_tensor_arg(X, "X").value,
-                                _tensor_arg(mask, "mask", torch.uint8).value,
-                                _tensor_arg(L, "L").value, _tensor_arg(E, "E").value,
-                                _tensor_arg(Y, "Y").value,
-                                _tensor_arg(mu, "mu", torch.float64).value, n1, n2, n3)
+        descs[i] = TpTensorDesc(_tensor_arg(X, "X"), _tensor_arg(mask, "mask", torch.uint8),
+                                _tensor_arg(L, "L"), _tensor_arg(E, "E"), _tensor_arg(Y, "Y"),
+                                _tensor_arg(mu, "mu", torch.float64), n1, n2, n3)
         dims += [n1, n2, n3]
     o = _opts(TP_OP_TCOMPLETE_SVT_BATCHED, dims, precision, status, max_sweeps)
     rc = lib().tcomplete_svt_batched(len(tensors), ctypes.cast(descs, ctypes.c_void_p), int(iters),
