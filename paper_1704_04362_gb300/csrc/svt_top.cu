@@ -712,6 +712,7 @@ __global__ void __launch_bounds__(32 * L) svt_top_coef_kernel(SvtTopArgs g, cons
                                                               const float* hi, int p,
                                                               int transpose) {
   __shared__ float coef[L];
+  __shared__ double nv_s[L], nh_s[L];
   const int f = blockIdx.x, q = g.q, lane = threadIdx.x & 31, j = threadIdx.x >> 5;
   if (!g.fast[f]) return;
   const float* Hr = hr + f * g.sG;
@@ -740,9 +741,16 @@ __global__ void __launch_bounds__(32 * L) svt_top_coef_kernel(SvtTopArgs g, cons
     nh += __shfl_xor_sync(0xffffffffu, nh, o);
   }
   if (lane == 0) {
+    nv_s[j] = nv;
+    nh_s[j] = nh;
+  }
+  __syncthreads();
+  if (threadIdx.x < L) {   // one warp's float64 divisions, not every warp's
+    nv = nv_s[lane];
+    nh = nh_s[lane];
     const double tau = 1.0 / *g.mu, sj = nv > 0.0 ? sqrt(nh / nv) : 0.0;
-    const bool up = (g.above[f] >> j) & 1u;
-    coef[j] = up && sj > tau ? float((sj - tau) / (sj * nv)) : 0.f;
+    const bool up = (g.above[f] >> lane) & 1u;
+    coef[lane] = up && sj > tau ? float((sj - tau) / (sj * nv)) : 0.f;
   }
   __syncthreads();
   float* Or = g.gr + f * g.sG;
