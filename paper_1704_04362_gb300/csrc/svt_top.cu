@@ -28,7 +28,7 @@
 // and 2 global loads per 16 packed FMAs) and by the certificate's panels, one
 // after the other, half the time each.
 // 41 slices of 144 x 256 (the 144 x 256 x 80 completion), one iteration: 3.5 ms
-// by the warm-started Jacobi and its GEMMs -> 0.61 ms here and 0.16 ms of GEMMs.
+// by the warm-started Jacobi and its GEMMs -> 0.61 ms here and 0.14 ms of GEMMs.
 // From 48 columns on (below, the Jacobi's slices are small and many fit an
 // SM) up to 384, where Q and Y (2 x 2 x 48 KB) still fit the shared memory.
 #include <algorithm>
@@ -40,7 +40,7 @@ namespace {
 
 constexpr int L = SVT_TOP_L;          // vectors kept per slice
 constexpr int LS = L + 1;             // row stride of the L x L matrices
-constexpr int MAX_WARPS = 24;
+constexpr int MAX_WARPS = 20;        // 96 registers a thread: eight loads of A in flight
 constexpr int MAX_ABOVE = L - 6;      // a buffer of vectors below the threshold
 constexpr int MAX_ROUNDS = 8;         // Rayleigh-Ritz rounds
 constexpr int RETRY = 4;              // iterations between attempts with too many above
@@ -58,13 +58,13 @@ struct Tile {   // one row, eight columns
 };
 
 // t += sum_k A(row, k) B[k][c0 .. c0+7]: A in global memory (column-major,
-// leading dimension lda), B in shared memory (row stride L).  The next four
+// leading dimension lda), B in shared memory (row stride L).  The next eight
 // values of A are loaded before the current ones are used.  (Two rows a thread
 // halve the loads of B but leave too few warps: 70 against 50 thousand cycles
 // for q = 144.)
 __device__ __forceinline__ void accumulate(Tile& t, const float* ar, const float* ai, int64_t lda,
                                            int K, const float* Br, const float* Bi, int c0) {
-  constexpr int U = 4;
+  constexpr int U = 8;
   float nr[U], ni_[U];
   auto fetch = [&](int k0) {
 #pragma unroll
@@ -409,25 +409,19 @@ __device__ bool certify(const Shared& s, float* gr, float* gi, int q, float unit
     __syncthreads();
     if (j0 + L < q) {   // rows below the block (nb == L here)
       const int lo = j0 + L;
-      Tile t[2];   // at most two row blocks per warp pair
-#pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        const int i0 = lo + ((warp >> 1) + w * nrw) * 16, ic = min(i0 + lr, q - 1);
-        t[w].clear();
-        if (i0 < q)
-          accumulate(t[w], gr + ic + int64_t(q) * j0, gi + ic + int64_t(q) * j0, q, L, s.Yr, s.Yi,
-                     c0);
-      }
-      __syncthreads();   // every row has been read
-#pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        const int i = lo + ((warp >> 1) + w * nrw) * 16 + lr;
+      for (int i0 = lo + (warp >> 1) * 16; i0 < q; i0 += nrw * 16) {
+        const int i = i0 + lr, ic = min(i, q - 1);
+        Tile t;
+        t.clear();
+        accumulate(t, gr + ic + int64_t(q) * j0, gi + ic + int64_t(q) * j0, q, L, s.Yr, s.Yi, c0);
+        // both warps of the pair (the column halves) have read these rows
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp >> 1)) : "memory");
         if (i >= q) continue;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int64_t o = i + int64_t(q) * (j0 + c0 + u);
-          gr[o] = column(t[w].re, u);
-          gi[o] = column(t[w].im, u);
+          gr[o] = column(t.re, u);
+          gi[o] = column(t.im, u);
         }
       }
     }
@@ -818,7 +812,7 @@ int svt_top_init(const SvtTopArgs& g, int64_t h, float* vr, float* vi, cudaStrea
 
 int svt_top_launch(const SvtTopArgs& g, int64_t h, cudaStream_t st) {
   const size_t smem = top_smem(g.q);
-  // two warps (the column halves) per 16 rows in as few passes as 24 warps
+  // two warps (the column halves) per 16 rows in as few passes as MAX_WARPS
   // allow, at least 16 for the small steps
   const int nrb = (g.q + 15) / 16, passes = (nrb + MAX_WARPS / 2 - 1) / (MAX_WARPS / 2);
   const int warps = std::max(2 * ((nrb + passes - 1) / passes), 16);
