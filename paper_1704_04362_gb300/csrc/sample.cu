@@ -264,7 +264,8 @@ __global__ void __launch_bounds__(256) draw_decide_kernel(
     int32_t* __restrict__ idx, float* __restrict__ scale, double* __restrict__ q_out) {
   const double total = draw_total(bpart, G, mode);
   const double cd = double(c);
-  for (int64_t j = int64_t(blockIdx.x) * 256 + threadIdx.x; j < n; j += int64_t(gridDim.x) * 256) {
+  for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
+       j += int64_t(gridDim.x) * blockDim.x) {
     double q = fmin(1.0, cd * draw_p(w, w2, mode, total, j));
     if (!(q > 0.0)) q = 0.0;   // also maps NaN to 0
     const uint64_t Q = uint64_t(q * 9007199254740992.0);   // floor(q 2^53), q in [0,1]
@@ -503,8 +504,13 @@ int launch_draw(const double* w, const double* w2, int64_t n, int64_t c, uint64_
       iid_weights_kernel<<<G, 256, 0, st>>>(w, w2, n, c, mode, bpart, G, W, sval, q_out);
       iid_draw_kernel<<<1, 1024, 0, st>>>(n, c, seed, stream_id, W, sval, idx, scale, count);
     } else {
-      draw_decide_kernel<<<G, 256, 0, st>>>(w, w2, n, c, seed, mode, stream_id, bpart, G, idx,
-                                            scale, q_out);
+      // float64 roots and divisions per index, two lanes a cycle and SM: up to
+      // 8192 indices in blocks of one warp, so that they spread over the chip
+      // (4000 indices: the three launches 23 -> 21 us); beyond, the
+      // blocks' own sums of bpart would cost more
+      const bool spread = n <= 8192;
+      draw_decide_kernel<<<spread ? unsigned((n + 31) / 32) : unsigned(G), spread ? 32 : 256, 0, st>>>(
+          w, w2, n, c, seed, mode, stream_id, bpart, G, idx, scale, q_out);
       draw_compact_kernel<<<1, 1024, 0, st>>>(n, idx, scale, count);
     }
   }
