@@ -17,13 +17,24 @@ namespace jrot {
 // and ||b'||^2 = beta + tg.
 __device__ __forceinline__ void rotation(float alpha, float beta, float gr, float gi, float g2,
                                          float& cs, float& sn, float& er, float& ei, float& tg) {
-  const float g = sqrtf(g2);
+  float g = sqrtf(g2);
+  er = gr / g;
+  ei = -gi / g;
+  if (g2 < 1e-30f) {
+    // g2 nears or leaves the normal range (null columns of a rank-deficient
+    // slice) and its root with it: gamma scaled by a power of two first, or
+    // e^{-i phi} is not of unit length and V loses its orthonormality
+    int e;
+    frexpf(fmaxf(fabsf(gr), fabsf(gi)), &e);
+    const float a = ldexpf(gr, -e), b = ldexpf(gi, -e), gs = sqrtf(a * a + b * b);
+    er = a / gs;
+    ei = -b / gs;
+    g = ldexpf(gs, e);
+  }
   const float zeta = (beta - alpha) / (2.f * g);
   const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
   cs = 1.f / sqrtf(1.f + t * t);
   sn = cs * t;
-  er = gr / g;
-  ei = -gi / g;
   tg = t * g;
 }
 __device__ __forceinline__ void rotation(float alpha, float beta, float gr, float gi, float g2,
@@ -50,14 +61,23 @@ __device__ __forceinline__ void rotation(double alpha, double beta, double gr, d
   e += (e & 1);                          // even, so that 2^(e/2) is exact
   const double sc = ldexp(1.0, -e);      // alpha, beta scaled to <= 1, g2 by sc^2
   const float af = float(alpha * sc), bf = float(beta * sc), g2f = float(g2 * sc * sc);
-  if (!(g2f > 1e-30f)) {   // |gamma| below float range after scaling: exact float64 path
-    const double g = sqrt(g2);
+  // outside float's range after scaling (|gamma| far below the norms, or norms
+  // kept through cancellation far below |gamma|): all in float64
+  if (!(g2f > 1e-30f && g2f < 1e30f) || g2 < 1e-290) {
+    double g = sqrt(g2);
+    er = gr / g;
+    ei = -gi / g;
+    if (g2 < 1e-290) {   // as in float32: gamma scaled before its square
+      frexp(fmax(fabs(gr), fabs(gi)), &e);
+      const double a = ldexp(gr, -e), b = ldexp(gi, -e), gs = sqrt(a * a + b * b);
+      er = a / gs;
+      ei = -b / gs;
+      g = ldexp(gs, e);
+    }
     const double zeta = (beta - alpha) / (2.0 * g);
     const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
     cs = 1.0 / sqrt(1.0 + t * t);
     sn = cs * t;
-    er = gr / g;
-    ei = -gi / g;
     tg = t * g;
     return;
   }
