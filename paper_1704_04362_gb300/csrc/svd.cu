@@ -29,6 +29,7 @@
 //      of singular values at the float32 rounding floor (rank-deficient
 //      input), which float32 cannot resolve.
 // Steps 2-3 are batched float64 GEMMs spread over all SMs.
+#include <algorithm>
 #include <atomic>
 
 #include "householder.cuh"
@@ -282,6 +283,20 @@ __device__ __forceinline__ int jpc_peek(const int* local, unsigned rank) {
   return v;
 }
 
+// the cluster address of CTA `rank`'s copy of `local`, and a 16-byte store to one
+__device__ __forceinline__ unsigned jpc_remote(const void* local, unsigned rank) {
+  const unsigned a = unsigned(__cvta_generic_to_shared(local));
+  unsigned remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(a), "r"(rank));
+  return remote;
+}
+
+__device__ __forceinline__ void jpc_store(unsigned remote, uint4 v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
 template <bool S, class T>
 __device__ __forceinline__ T jld(const T* x) {
   if constexpr (S) return *x;
@@ -350,6 +365,66 @@ __device__ __forceinline__ bool jpc_pair(T* ar, T* ai, T* br, T* bi, T* var, T* 
     jst<S>(vbr + r, sn * xr + cs * yr);
     jst<S>(vbi + r, sn * xi + cs * yi);
   }
+  return true;
+}
+
+// jpc_pair<true, float> for columns of up to 32 R values, each lane's rows held
+// in registers from the inner products to the rotation (V's are loaded while
+// the sums and the angle are formed): the same operations in the same order.
+template <int R>
+__device__ __forceinline__ bool jpc_pair_reg(float* ar, float* ai, float* br, float* bi, float* var,
+                                             float* vai, float* vbr, float* vbi, int p, int q,
+                                             int lane, float tol) {
+  float xr[R], xi[R], yr[R], yi[R], ur[R], ui[R], wr[R], wi[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int r = lane + 32 * k;
+    const bool in = r < p;
+    xr[k] = in ? ar[r] : 0.f;
+    xi[k] = in ? ai[r] : 0.f;
+    yr[k] = in ? br[r] : 0.f;
+    yi[k] = in ? bi[r] : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int r = lane + 32 * k;
+    const bool in = r < q;
+    ur[k] = in ? var[r] : 0.f;
+    ui[k] = in ? vai[r] : 0.f;
+    wr[k] = in ? vbr[r] : 0.f;
+    wi[k] = in ? vbi[r] : 0.f;
+  }
+  float alpha = 0, beta = 0, gr = 0, gi = 0;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    alpha += xr[k] * xr[k] + xi[k] * xi[k];
+    beta += yr[k] * yr[k] + yi[k] * yi[k];
+    gr += xr[k] * yr[k] + xi[k] * yi[k];
+    gi += xr[k] * yi[k] - xi[k] * yr[k];
+  }
+  alpha = warp_sum_t(alpha);
+  beta = warp_sum_t(beta);
+  gr = warp_sum_t(gr);
+  gi = warp_sum_t(gi);
+  const float g2 = gr * gr + gi * gi;
+  if (!(g2 > tol * tol * alpha * beta) || g2 == 0.f) return false;
+  float cs, sn, er, ei, tg;
+  rotation(alpha, beta, gr, gi, g2, cs, sn, er, ei, tg);
+  auto rotate = [&](float* a, float* b, float* c, float* d, const float* x, const float* x2,
+                    const float* y, const float* y2, int n) {
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int r = lane + 32 * k;
+      if (r >= n) continue;
+      const float tr = y[k] * er - y2[k] * ei, ti = y[k] * ei + y2[k] * er;
+      a[r] = cs * x[k] - sn * tr;
+      b[r] = cs * x2[k] - sn * ti;
+      c[r] = sn * x[k] + cs * tr;
+      d[r] = sn * x2[k] + cs * ti;
+    }
+  };
+  rotate(ar, ai, br, bi, xr, xi, yr, yi, p);
+  rotate(var, vai, vbr, vbi, ur, ui, wr, wi, q);
   return true;
 }
 
@@ -558,6 +633,214 @@ __global__ void __cluster_dims__(JPC, 1, 1) __launch_bounds__(JPC_THREADS)
         xr[r] = __ldcg(xr + r) * inv;
         xi[r] = __ldcg(xi + r) * inv;
       }
+    }
+  }
+}
+
+// ---- the same with the columns kept in the cluster's shared memories ----
+//
+// Where two block pairs fit (RING), G, V and the norms never leave the cluster
+// between rounds: a CTA rotates the pair in one buffer, then pushes each block
+// into the other buffer of the CTA that owns it in the next round (stores to
+// the cluster's shared memory), and one cluster barrier ends the round.  The
+// pairs, their order and their arithmetic are jacobi_cluster_kernel's, so the
+// results are the same.  A round through L2 is bound by the copies'
+// latency and the fence before its barrier, not by the rotations: 9 slices of
+// 64 x 48 in float32 0.561 -> 0.436 ms a call, 0.36 with the columns of a pair in
+// registers between its inner products and its rotation (jpc_pair_reg).
+
+// Values of one block (bs columns of G, V and the norms) in a buffer: G re, G
+// im, V re, V im, norms; a multiple of 16 bytes.
+template <class T>
+__host__ __device__ __forceinline__ int jpc_block_vals(int p, int q) {
+  const int bs = (q + JPC_BLOCKS - 1) / JPC_BLOCKS, n = bs * (2 * (p + q) + 1);
+  constexpr int V = 16 / int(sizeof(T));
+  return (n + V - 1) / V * V;
+}
+
+template <class T>
+size_t jacobi_ring_smem(int p, int q) {
+  const size_t bytes = 4 * size_t(jpc_block_vals<T>(p, q)) * sizeof(T);
+  return bytes <= size_t(200) * 1024 ? bytes : 0;
+}
+
+// CTA and slot (0: I, 1: J) of block B in a round.
+__device__ __forceinline__ int jpc_owner(int B, int round, int& slot) {
+  constexpr int n = JPC_BLOCKS - 1;
+  slot = B == round;
+  if (B == n || B == round) return 0;
+  const int up = (B - round + n) % n;
+  slot = up > n / 2;
+  return slot ? n - up : up;
+}
+
+// R: rows a lane holds (p, q <= 32 R, float32), or 0.
+template <class T, int R>
+__global__ void __cluster_dims__(JPC, 1, 1) __launch_bounds__(JPC_THREADS, 1)
+    jacobi_ring_kernel(T* g_re, T* g_im, int64_t sG, T* v_re, T* v_im, int64_t sV, T* sig, int p,
+                       int q, int max_sweeps, const int* real_flags, int32_t* status, int flags,
+                       const int* skip) {
+  extern __shared__ __align__(16) unsigned char jpc_smem[];
+  constexpr bool keep = sizeof(T) == 8;
+  const int c = int(jpc_rank());
+  const int64_t b = blockIdx.x / JPC;
+  if (skip && skip[b]) return;   // the whole cluster: this slice needs no vectors
+  T* const Gr = g_re + b * sG;
+  T* const Gi = g_im + b * sG;
+  T* const Vr = v_re + b * sV;
+  T* const Vi = v_im + b * sV;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = JPC_THREADS / 32;
+  const int bs = (q + JPC_BLOCKS - 1) / JPC_BLOCKS;
+  const int bs2 = bs + (bs & 1);   // positions of the internal round-robin
+  const int bv = jpc_block_vals<T>(p, q);
+  T* const sm = reinterpret_cast<T*>(jpc_smem);   // [buffer][slot][bv]
+  __shared__ int rotated, any_s;
+  const bool real = real_flags ? real_flags[b] != 0 : false;
+  auto block_of = [&](int round, int slot) {
+    if (c == 0) return slot ? round : JPC_BLOCKS - 1;
+    return slot ? (round - c + JPC_BLOCKS - 1) % (JPC_BLOCKS - 1) : (round + c) % (JPC_BLOCKS - 1);
+  };
+  // a block's arrays
+  auto gre = [&](T* blk) { return blk; };
+  auto gim = [&](T* blk) { return blk + bs * p; };
+  auto vre = [&](T* blk) { return blk + 2 * bs * p; };
+  auto vim = [&](T* blk) { return blk + 2 * bs * p + bs * q; };
+  auto nrm = [&](T* blk) { return blk + 2 * bs * (p + q); };
+
+  for (int slot = 0; slot < 2; ++slot) {
+    T* blk = sm + slot * bv;
+    const int g0 = block_of(0, slot) * bs;
+    for (int l = warp; l < bs && g0 + l < q; l += nw) {
+      const int64_t j = g0 + l;
+      for (int r = lane; r < p; r += 32) {
+        gre(blk)[l * p + r] = Gr[j * p + r];
+        gim(blk)[l * p + r] = real ? T(0) : Gi[j * p + r];
+      }
+      for (int r = lane; r < q; r += 32) {
+        const bool init = flags & JAC_INIT_V;
+        vre(blk)[l * q + r] = init ? (r == j ? T(1) : T(0)) : Vr[j * q + r];
+        vim(blk)[l * q + r] = init || real ? T(0) : Vi[j * q + r];
+      }
+    }
+  }
+  T tol = T(8) * Eps<T>::v * sqrt(T(p));
+  if (tol < T(keep ? 1e-13 : 1e-6)) tol = T(keep ? 1e-13 : 1e-6);
+  jpc_cluster_sync();   // also: every CTA of the cluster runs, so its memory may be written
+
+  int buf = 0, sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    if (tid == 0) rotated = 0;
+    if (keep) {
+      for (int k = warp; k < 2 * bs; k += nw) {
+        T* blk = sm + (2 * buf + (k >= bs)) * bv;
+        const int l = k >= bs ? k - bs : k;
+        if (block_of(0, k >= bs) * bs + l >= q) continue;
+        const T* xr = gre(blk) + l * p;
+        const T* xi = gim(blk) + l * p;
+        T acc = 0;
+        for (int r = lane; r < p; r += 32) acc += xr[r] * xr[r] + xi[r] * xi[r];
+        acc = warp_sum_t(acc);
+        if (lane == 0) nrm(blk)[l] = acc;
+      }
+    }
+    __syncthreads();
+    bool rot = false;
+    for (int round = 0; round < JPC_BLOCKS - 1; ++round, buf ^= 1) {
+      T* const A = sm + 2 * buf * bv;
+      const int i0 = block_of(round, 0) * bs, j0 = block_of(round, 1) * bs;
+      auto gcol = [&](int l) { return l < bs ? i0 + l : j0 + l - bs; };
+      // rotates local columns (la, lb) of the block pair
+      auto pair = [&](int la, int lb) {
+        int ga = gcol(la), gb = gcol(lb);
+        if (ga >= q || gb >= q) return;
+        if (ga > gb) {
+          const int t = la; la = lb; lb = t;
+        }
+        T* const x = A + (la < bs ? 0 : bv);
+        T* const y = A + (lb < bs ? 0 : bv);
+        la = la < bs ? la : la - bs;
+        lb = lb < bs ? lb : lb - bs;
+        if constexpr (R > 0)
+          rot |= jpc_pair_reg<R>(gre(x) + la * p, gim(x) + la * p, gre(y) + lb * p,
+                                 gim(y) + lb * p, vre(x) + la * q, vim(x) + la * q,
+                                 vre(y) + lb * q, vim(y) + lb * q, p, q, lane, tol);
+        else
+          rot |= jpc_pair<true, T>(gre(x) + la * p, gim(x) + la * p, gre(y) + lb * p,
+                                   gim(y) + lb * p, vre(x) + la * q, vim(x) + la * q,
+                                   vre(y) + lb * q, vim(y) + lb * q, nrm(x) + la, nrm(y) + lb, p,
+                                   q, lane, tol);
+      };
+      if (round == 0) {
+        // internal pairs of both blocks: bs2 - 1 steps of bs2 / 2 pairs each
+        for (int step = 0; step < bs2 - 1; ++step) {
+          for (int k = warp; k < bs2; k += nw) {
+            const int off = k < bs2 / 2 ? 0 : bs;
+            const int i = k < bs2 / 2 ? k : k - bs2 / 2;
+            int x, y;
+            if (i == 0) {
+              x = bs2 - 1;
+              y = step;
+            } else {
+              x = (step + i) % (bs2 - 1);
+              y = (step - i + bs2 - 1) % (bs2 - 1);
+            }
+            if (x < bs && y < bs) pair(off + x, off + y);
+          }
+          __syncthreads();
+        }
+      }
+      // cross pairs: step t pairs column i of block I with (i + t) mod bs of J
+      for (int t = 0; t < bs; ++t) {
+        for (int i = warp; i < bs; i += nw) pair(i, bs + (i + t < bs ? i + t : i + t - bs));
+        __syncthreads();
+      }
+      // both blocks to their owners of the next round
+      const int next = round + 1 < JPC_BLOCKS - 1 ? round + 1 : 0;
+      constexpr int V = 16 / int(sizeof(T));
+      const int nv = bv / V;
+      unsigned dst[2];
+#pragma unroll
+      for (int slot = 0; slot < 2; ++slot) {
+        int to_slot;
+        const int to = jpc_owner(block_of(round, slot), next, to_slot);
+        dst[slot] = jpc_remote(sm + (2 * (buf ^ 1) + to_slot) * bv, unsigned(to));
+      }
+      const uint4* from = reinterpret_cast<const uint4*>(A);   // both blocks, one after the other
+      for (int e = tid; e < 2 * nv; e += JPC_THREADS)
+        jpc_store(e < nv ? dst[0] + 16u * unsigned(e) : dst[1] + 16u * unsigned(e - nv), from[e]);
+      if (rot && lane == 0) rotated = 1;
+      jpc_cluster_sync();
+    }
+    if (tid == 0) {
+      int any = 0;
+      for (int r = 0; r < JPC; ++r) any |= jpc_peek(&rotated, unsigned(r));
+      any_s = any;
+    }
+    jpc_cluster_sync();   // every CTA has read every flag before any resets its own
+    if (!any_s) break;
+  }
+  if (sweep >= max_sweeps && c == 0 && tid == 0 && status) atomicOr(status, TP_DEV_NOCONV);
+  // singular values and the columns (optionally of unit length)
+  for (int k = warp; k < 2 * bs; k += nw) {
+    const int slot = k >= bs, l = slot ? k - bs : k;
+    const int64_t j = block_of(0, slot) * bs + l;
+    if (j >= q) continue;
+    T* blk = sm + (2 * buf + slot) * bv;
+    const T* xr = gre(blk) + l * p;
+    const T* xi = gim(blk) + l * p;
+    T acc = 0;
+    for (int r = lane; r < p; r += 32) acc += xr[r] * xr[r] + xi[r] * xi[r];
+    const T s = sqrt(warp_sum_t(acc));
+    if (lane == 0) sig[b * q + j] = s;
+    const T inv = s > T(0) ? T(1) / s : T(0);
+    const bool unit = flags & JAC_NORMALIZE;
+    for (int r = lane; r < p; r += 32) {
+      Gr[j * p + r] = unit ? xr[r] * inv : xr[r];
+      Gi[j * p + r] = unit ? xi[r] * inv : xi[r];
+    }
+    for (int r = lane; r < q; r += 32) {
+      Vr[j * q + r] = vre(blk)[l * q + r];
+      Vi[j * q + r] = vim(blk)[l * q + r];
     }
   }
 }
@@ -797,11 +1080,19 @@ int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T*
                           int32_t* status, int flags, cudaStream_t st,
                           const int* skip = nullptr) {
   if (batch <= 0 || q <= 0) return TP_OK;
-  const size_t smem = jacobi_cluster_smem<T>(p, q);
+  const size_t smem = jacobi_cluster_smem<T>(p, q), ring = jacobi_ring_smem<T>(p, q);
   const unsigned grid = unsigned(batch) * JPC;
   {
     KernelScope ks(sizeof(T) == 4 ? "jacobi_f32" : "jacobi_svd", st);
-    if (smem) {
+    if (ring) {
+      constexpr bool f32 = sizeof(T) == 4;
+      auto kernel = f32 && std::max(p, q) <= 64    ? jacobi_ring_kernel<T, f32 ? 2 : 0>
+                    : f32 && std::max(p, q) <= 128 ? jacobi_ring_kernel<T, f32 ? 4 : 0>
+                                                   : jacobi_ring_kernel<T, 0>;
+      TP_SET_SMEM(kernel, ring);
+      kernel<<<grid, JPC_THREADS, ring, st>>>(gr, gi, sG, vr, vi, sV, sig, p, q, max_sweeps,
+                                              real_flags, status, flags, skip);
+    } else if (smem) {
       if (int rc = set_smem_attr((const void*)jacobi_cluster_kernel<T, true>, smem,
                                  "jacobi_cluster_kernel"))
         return rc;
