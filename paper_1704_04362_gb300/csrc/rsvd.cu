@@ -54,20 +54,17 @@ __global__ void conj_transpose_kernel(const float* __restrict__ ir, const float*
   }
 }
 
-// Split operand planes (tensor-core products) of a batch of column-major
-// complex matrices: element (r, c) of matrix f (rows x cols, at
-// f*s_src + r + ld_src*c) goes to f*s_dst + r + ld_dst*c of the hi/lo
-// planes (3xTF32 float or BF16x3 bf16 pairs), the imaginary part negated
-// when conj; rows [rows, ld_dst) are zero (the K padding of the tiles).
-// The split planes of X_hat transposed without conjugation, for the
-// tensor-core products X_hat B: element (i, j) of X_hat (n1 x n2,
-// column-major) goes to j + ldk i of each plane (K-major, rows j from n2 to
-// ldk zero), through a 32 x 32 shared-memory tile as conj_transpose_kernel
-// moves it.
+// The split planes of X_hat for the tensor-core products X_hat B and X_hat^H B,
+// from one read of X_hat (n1 x n2, column-major) through 32 x 32 shared-memory
+// tiles: element (i, j) goes to j + ldk i of A's planes (K-major, rows j from n2
+// to ldk zero) and, conjugated, to i + ldh j of H's (rows i from n1 to ldh
+// zero).  Both together 0.16 -> 0.10 ms on 1001 slices of 128 x 128.
+struct SplitPlanes {
+  float *re_hi, *re_lo, *im_hi, *im_lo;
+};
 __global__ void transpose_split_kernel(const float* __restrict__ ir, const float* __restrict__ ii,
-                                       int64_t n1, int64_t n2, int64_t ldk, int bf16,
-                                       float* __restrict__ re_hi, float* __restrict__ re_lo,
-                                       float* __restrict__ im_hi, float* __restrict__ im_lo) {
+                                       int64_t n1, int64_t n2, int64_t ldk, int64_t ldh, int bf16,
+                                       SplitPlanes A, SplitPlanes H) {
   __shared__ float tr[32][33], ti[32][33];
   const int64_t f = blockIdx.z;
   const int64_t i0 = int64_t(blockIdx.x) * 32, j0 = int64_t(blockIdx.y) * 32;
@@ -76,23 +73,34 @@ __global__ void transpose_split_kernel(const float* __restrict__ ir, const float
   for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
     const int64_t i = i0 + threadIdx.x, j = j0 + dy;
     const bool in = i < n1 && j < n2;
-    tr[dy][threadIdx.x] = in ? sr[i + n1 * j] : 0.f;
-    ti[dy][threadIdx.x] = in ? si[i + n1 * j] : 0.f;
+    const float re = in ? sr[i + n1 * j] : 0.f, im = in ? si[i + n1 * j] : 0.f;
+    tr[dy][threadIdx.x] = re;
+    ti[dy][threadIdx.x] = im;
+    if (i < ldh && j < n2) {
+      const int64_t o = f * ldh * n2 + i + ldh * j;
+      dftc::put_split(H.re_hi, H.re_lo, bf16 != 0, o, re);
+      dftc::put_split(H.im_hi, H.im_lo, bf16 != 0, o, -im);
+    }
   }
   __syncthreads();
   for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
     const int64_t j = j0 + threadIdx.x, i = i0 + dy;
     if (i < n1 && j < ldk) {
       const int64_t o = f * ldk * n1 + j + ldk * i;
-      dftc::put_split(re_hi, re_lo, bf16 != 0, o, tr[threadIdx.x][dy]);
-      dftc::put_split(im_hi, im_lo, bf16 != 0, o, ti[threadIdx.x][dy]);
+      dftc::put_split(A.re_hi, A.re_lo, bf16 != 0, o, tr[threadIdx.x][dy]);
+      dftc::put_split(A.im_hi, A.im_lo, bf16 != 0, o, ti[threadIdx.x][dy]);
     }
   }
 }
 
+// Split operand planes (tensor-core products) of a batch of column-major
+// complex matrices: element (r, c) of matrix f (rows x cols, at
+// f*s_src + r + ld_src*c) goes to f*s_dst + r + ld_dst*c of the hi/lo
+// planes (3xTF32 float or BF16x3 bf16 pairs); rows [rows, ld_dst) are zero (the
+// K padding of the tiles).
 __global__ void split_planes_kernel(const float* __restrict__ sr, const float* __restrict__ si,
                                     int64_t rows, int64_t cols, int64_t ld_src, int64_t s_src,
-                                    int64_t h, int64_t ld_dst, int64_t s_dst, int conj, int bf16,
+                                    int64_t h, int64_t ld_dst, int64_t s_dst, int bf16,
                                     float* __restrict__ re_hi, float* __restrict__ re_lo,
                                     float* __restrict__ im_hi, float* __restrict__ im_lo) {
   const int64_t per = ld_dst * cols, total = per * h;
@@ -104,7 +112,6 @@ __global__ void split_planes_kernel(const float* __restrict__ sr, const float* _
     if (r < rows) {
       vr = sr[f * s_src + r + ld_src * c];
       vi = si[f * s_src + r + ld_src * c];
-      if (conj) vi = -vi;
     }
     const int64_t o = f * s_dst + r + ld_dst * c;
     dftc::put_split(re_hi, re_lo, bf16 != 0, o, vr);
@@ -287,8 +294,9 @@ __device__ void tridiag_form_q(const float2* G, float2* W, int l, int ls, const 
 // Eigenvalues of the real symmetric tridiagonal (d, e) -- d[i * stride],
 // e[i * stride], e[l-1] = 0 -- by the implicit QL algorithm with
 // Wilkinson's shift from the leading 2 x 2 (Bowdler, Martin, Reinsch and
-// Wilkinson, 1968), run by one thread: each chase goes from the bottom of
-// the unreduced block to its top, deflating off-diagonals below
+// Wilkinson, 1968), run by one warp, whose lanes together search for the end of
+// the unreduced block (one thread's search was a fifth of the kernel) and whose
+// lane 0 chases: each chase goes from the bottom of the unreduced block to its top, deflating off-diagonals below
 // FLT_EPSILON (|d_m| + |d_m+1|), and its plane rotations are appended to
 // log (at most cap; rotation i mixes columns i and i + 1, code i, or
 // -(i + 1) for a chase's first rotation).  T is first scaled by a power of
@@ -303,26 +311,33 @@ struct QlRot {
 };
 
 __device__ bool ql_chase(float* __restrict__ d, float* __restrict__ e, int stride, int l,
-                         QlRot* __restrict__ log, int cap, int max_iter, int* count) {
+                         QlRot* __restrict__ log, int cap, int max_iter, int lane, int* count) {
 #define D(i) d[(i) * stride]
 #define E(i) e[(i) * stride]
   float mx = 0.f;
-  for (int i = 0; i < l; ++i) mx = fmaxf(mx, fmaxf(fabsf(D(i)), fabsf(E(i))));
+  for (int i = lane; i < l; i += 32) mx = fmaxf(mx, fmaxf(fabsf(D(i)), fabsf(E(i))));
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (mx > 0.f && isfinite(mx)) {
     int ex;
     frexpf(mx, &ex);
-    for (int i = 0; i < l; ++i) {
+    for (int i = lane; i < l; i += 32) {
       D(i) = ldexpf(D(i), -ex);
       E(i) = ldexpf(E(i), -ex);
     }
   }
+  __syncwarp();
   bool ok = true;
   int cnt = 0, l0 = 0, it = 0;
   while (l0 < l) {
     int m = l0;
-    for (; m + 1 < l; ++m) {
-      const float dd = fabsf(D(m)) + fabsf(D(m + 1));
-      if (fabsf(E(m)) <= FLT_EPSILON * dd) break;
+    for (;; m += 32) {
+      const int t = m + lane;
+      const bool end = t + 1 >= l || fabsf(E(t)) <= FLT_EPSILON * (fabsf(D(t)) + fabsf(D(t + 1)));
+      const unsigned ends = __ballot_sync(0xffffffffu, end);
+      if (ends) {
+        m += __ffs(ends) - 1;
+        break;
+      }
     }
     if (m == l0) {
       ++l0;
@@ -331,61 +346,66 @@ __device__ bool ql_chase(float* __restrict__ d, float* __restrict__ e, int strid
     }
     if (cnt + (m - l0) > cap || ++it > max_iter) {
       ok = false;
-      E(l0) = 0.f;
+      if (lane == 0) E(l0) = 0.f;
+      __syncwarp();
       continue;
     }
-    float g = (D(l0 + 1) - D(l0)) / (2.f * E(l0));
-    const float r0 = hypotf(g, 1.f);
-    g = D(m) - D(l0) + E(l0) / (g + copysignf(r0, g));
-    float s = 1.f, c = 1.f, pp = 0.f;
-    float dn = D(m);   // d[i + 1] of the step below, carried
-    bool early = false;
-    // e[i] and d[i] of the next step are loaded a step ahead (a step writes
-    // only index i + 1), off the chain of dependent arithmetic
-    float ei_n = E(m - 1), di_n = D(m - 1);
-    for (int i = m - 1; i >= l0; --i) {
-      const float ei = ei_n, di = di_n;
-      if (i > l0) {
-        ei_n = E(i - 1);
-        di_n = D(i - 1);
+    if (lane == 0) {
+      float g = (D(l0 + 1) - D(l0)) / (2.f * E(l0));
+      const float r0 = hypotf(g, 1.f);
+      g = D(m) - D(l0) + E(l0) / (g + copysignf(r0, g));
+      float s = 1.f, c = 1.f, pp = 0.f;
+      float dn = D(m);   // d[i + 1] of the step below, carried
+      bool early = false;
+      // e[i] and d[i] of the next step are loaded a step ahead (a step writes
+      // only index i + 1), off the chain of dependent arithmetic
+      float ei_n = E(m - 1), di_n = D(m - 1);
+      for (int i = m - 1; i >= l0; --i) {
+        const float ei = ei_n, di = di_n;
+        if (i > l0) {
+          ei_n = E(i - 1);
+          di_n = D(i - 1);
+        }
+        const float f = s * ei, b = c * ei;
+        // r = sqrt(f^2 + g^2) and 1/r from the hardware reciprocal square root
+        // refined by one Newton-Raphson step y (3 - x y^2) / 2 (subnormal x:
+        // the rounded square root and reciprocal)
+        const float x = fmaf(f, f, g * g);
+        float r, inv;
+        if (x >= FLT_MIN) {
+          float y = rsqrtf(x);
+          y *= fmaf(-0.5f * x, y * y, 1.5f);
+          inv = y;
+          r = x * y;
+        } else {
+          r = sqrtf(x);
+          inv = r > 0.f ? __frcp_rn(r) : 0.f;
+        }
+        E(i + 1) = r;
+        if (r == 0.f) {   // the chase splits: restart from the new block
+          D(i + 1) = dn - pp;
+          E(m) = 0.f;
+          early = true;
+          break;
+        }
+        s = f * inv;
+        c = g * inv;
+        g = dn - pp;
+        r = fmaf(di - g, s, 2.f * c * b);
+        pp = s * r;
+        D(i + 1) = g + pp;
+        g = fmaf(c, r, -b);
+        dn = di;
+        log[cnt++] = QlRot{i == m - 1 ? -(i + 1) : i, c, s};
       }
-      const float f = s * ei, b = c * ei;
-      // r = sqrt(f^2 + g^2) and 1/r from the hardware reciprocal square root
-      // refined by one Newton-Raphson step y (3 - x y^2) / 2 (subnormal x:
-      // the rounded square root and reciprocal)
-      const float x = fmaf(f, f, g * g);
-      float r, inv;
-      if (x >= FLT_MIN) {
-        float y = rsqrtf(x);
-        y *= fmaf(-0.5f * x, y * y, 1.5f);
-        inv = y;
-        r = x * y;
-      } else {
-        r = sqrtf(x);
-        inv = r > 0.f ? __frcp_rn(r) : 0.f;
-      }
-      E(i + 1) = r;
-      if (r == 0.f) {   // the chase splits: restart from the new block
-        D(i + 1) = dn - pp;
+      if (!early) {
+        D(l0) = D(l0) - pp;
+        E(l0) = g;
         E(m) = 0.f;
-        early = true;
-        break;
       }
-      s = f * inv;
-      c = g * inv;
-      g = dn - pp;
-      r = fmaf(di - g, s, 2.f * c * b);
-      pp = s * r;
-      D(i + 1) = g + pp;
-      g = fmaf(c, r, -b);
-      dn = di;
-      log[cnt++] = QlRot{i == m - 1 ? -(i + 1) : i, c, s};
     }
-    if (!early) {
-      D(l0) = D(l0) - pp;
-      E(l0) = g;
-      E(m) = 0.f;
-    }
+    cnt = __shfl_sync(0xffffffffu, cnt, 0);
+    __syncwarp();
   }
 #undef D
 #undef E
@@ -405,10 +425,36 @@ __device__ __forceinline__ void ql_replay(float2* W, int l, int ls,
   // W(r, i), component t & 1 of row r = t >> 1, at float index 2 ls i + t
   float* __restrict__ z = reinterpret_cast<float*>(W) + threadIdx.x;
   const int cs = 2 * ls;
-#pragma unroll 4
-  for (int q = 0; q < cnt; ++q) {
+  // Within a chase the columns descend one by one, so the next eight values are
+  // loaded before the eight dependent rotations store theirs (one by one, every
+  // load waited for the store before it).
+  constexpr int U = 8;
+  int q = 0;
+  while (q < cnt) {
     const QlRot R = log[q];
     const int i = R.code < 0 ? -R.code - 1 : R.code;
+    if (R.code >= 0 && q + U <= cnt) {
+      QlRot r[U];
+      float x[U];
+      bool run = true;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        r[u] = log[q + u];
+        run = run && r[u].code == i - u;
+      }
+      if (run) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = z[cs * (i - u)];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          z[cs * (i - u + 1)] = fmaf(r[u].s, x[u], r[u].c * carry);
+          carry = fmaf(r[u].c, x[u], -r[u].s * carry);
+        }
+        prev = i - (U - 1);
+        q += U;
+        continue;
+      }
+    }
     if (R.code < 0) {   // a new chase: the previous one's last column first
       if (prev >= 0) z[cs * prev] = carry;
       carry = z[cs * (i + 1)];
@@ -417,6 +463,7 @@ __device__ __forceinline__ void ql_replay(float2* W, int l, int ls,
     z[cs * (i + 1)] = fmaf(R.s, zi, R.c * carry);
     carry = fmaf(R.c, zi, -R.s * carry);
     prev = i;
+    ++q;
   }
 }
 __device__ __forceinline__ void ql_replay_end(float2* W, int l, int ls, int prev, float carry) {
@@ -525,21 +572,46 @@ __global__ void __launch_bounds__(QL_THREADS) core_ql_kernel(
     QlRot* __restrict__ log, int32_t* __restrict__ log_count, int max_iter, int32_t* status) {
   extern __shared__ float qsm[];   // d (l), e (l)
   const int64_t f = blockIdx.x;
-  if (threadIdx.x != 0) return;
+  const int lane = threadIdx.x;
   float* d = qsm;
   float* e = qsm + l;
-  for (int i = 0; i < l; ++i) {
+  for (int i = lane; i < l; i += 32) {
     d[i] = d_in[f * l + i];
     e[i] = i + 1 < l ? e_in[f * l + i] : 0.f;
   }
   const int cap = QL_LOG_PER_L * l;
   int cnt = 0;
-  const bool ok = ql_chase(d, e, 1, l, log + f * cap, cap, max_iter, &cnt);
-  log_count[f] = cnt;
-  if (!ok && status) atomicOr(status, TP_DEV_NOCONV);
+  __syncwarp();
+  const bool ok = ql_chase(d, e, 1, l, log + f * cap, cap, max_iter, lane, &cnt);
+  if (lane == 0) log_count[f] = cnt;
+  if (!ok && lane == 0 && status) atomicOr(status, TP_DEV_NOCONV);
 }
 
 constexpr int FIN_RB = 64;   // rows of B^H staged per step of P = B^H W
+constexpr int FIN_NC = 4;    // columns of W a warp takes at once
+
+// Two rows (lane, lane + 32) of the staged block times FIN_NC columns of W (at
+// wc[u]): the rows' values are read once for all the columns.  Rows past the
+// block's end give values that nobody stores.  (A column at a time was bound by
+// its two shared-memory loads per four multiply-adds: core_finish 0.61 ->
+// 0.565 ms on 1001 slices of 128 x 50, the replay in blocks of eight included.)
+__device__ __forceinline__ void fin_product(const float2* stage, const float2* const (&wc)[FIN_NC],
+                                            int l, int lane, float2 (&out)[2][FIN_NC]) {
+#pragma unroll
+  for (int u = 0; u < FIN_NC; ++u) out[0][u] = out[1][u] = make_float2(0.f, 0.f);
+#pragma unroll 2
+  for (int m = 0; m < l; ++m) {
+    const float2 b0 = stage[m * FIN_RB + lane], b1 = stage[m * FIN_RB + lane + 32];
+#pragma unroll
+    for (int u = 0; u < FIN_NC; ++u) {
+      const float2 w = wc[u][m], v = make_float2(w.y, w.x);
+      out[0][u] = __ffma2_rn(make_float2(-b0.y, b0.y), v, out[0][u]);
+      out[0][u] = __ffma2_rn(make_float2(b0.x, b0.x), w, out[0][u]);
+      out[1][u] = __ffma2_rn(make_float2(-b1.y, b1.y), v, out[1][u]);
+      out[1][u] = __ffma2_rn(make_float2(b1.x, b1.x), w, out[1][u]);
+    }
+  }
+}
 
 __global__ void __launch_bounds__(EIG_THREADS) core_finish_kernel(
     const float* __restrict__ bh_re, const float* __restrict__ bh_im, int p, int l, int k,
@@ -593,22 +665,28 @@ __global__ void __launch_bounds__(EIG_THREADS) core_finish_kernel(
                                            __ldg(bi + r0 + rr + int64_t(p) * m));
     }
     __syncthreads();
-    for (int j = warp; j < l; j += nwarp) {
-      const float2* wj = Wf + j * ls;
-      double acc = 0.0;
-      for (int rr = lane; rr < nr; rr += 32) {
-        float pr = 0.f, pim = 0.f;
-        for (int m = 0; m < l; ++m) {
-          const float2 b = stage[m * FIN_RB + rr];
-          const float2 w = wj[m];
-          pr = fmaf(b.x, w.x, fmaf(-b.y, w.y, pr));
-          pim = fmaf(b.x, w.y, fmaf(b.y, w.x, pim));
+    for (int j0 = FIN_NC * warp; j0 < l; j0 += FIN_NC * nwarp) {
+      const float2* wc[FIN_NC];
+#pragma unroll
+      for (int u = 0; u < FIN_NC; ++u) wc[u] = Wf + min(j0 + u, l - 1) * ls;
+      float2 out[2][FIN_NC];
+      fin_product(stage, wc, l, lane, out);
+#pragma unroll
+      for (int u = 0; u < FIN_NC; ++u) {
+        const int j = j0 + u;
+        if (j >= l) break;
+        double acc = 0.0;
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          const int rr = lane + 32 * w;
+          if (rr >= nr) break;
+          const float2 v = out[w][u];
+          P[r0 + rr + int64_t(p) * j] = v;
+          acc += double(v.x) * v.x + double(v.y) * v.y;
         }
-        P[r0 + rr + int64_t(p) * j] = make_float2(pr, pim);
-        acc += double(pr) * pr + double(pim) * pim;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) sig2[j] += acc;   // column j belongs to this warp in every chunk
       }
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) sig2[j] += acc;   // column j belongs to this warp in every chunk
     }
   }
   __syncthreads();
@@ -660,19 +738,24 @@ __global__ void __launch_bounds__(EIG_THREADS) core_finish_kernel(
                                              __ldg(qif + r0 + rr + int64_t(n1) * m));
       }
       __syncthreads();
-      for (int c = warp; c < k; c += nwarp) {
-        const float2* wj = Wf + order[c] * ls;
-        for (int rr = lane; rr < nr; rr += 32) {
-          float pr = 0.f, pim = 0.f;
-          if (c < kr)
-            for (int m = 0; m < l; ++m) {
-              const float2 q = stage[m * FIN_RB + rr];
-              const float2 w = wj[m];
-              pr = fmaf(q.x, w.x, fmaf(-q.y, w.y, pr));
-              pim = fmaf(q.x, w.y, fmaf(q.y, w.x, pim));
-            }
-          ur[f * int64_t(n1) * k + r0 + rr + int64_t(n1) * c] = pr;
-          ui[f * int64_t(n1) * k + r0 + rr + int64_t(n1) * c] = pim;
+      for (int c0 = FIN_NC * warp; c0 < k; c0 += FIN_NC * nwarp) {
+        const float2* wc[FIN_NC];
+#pragma unroll
+        for (int u = 0; u < FIN_NC; ++u) wc[u] = Wf + order[min(c0 + u, k - 1)] * ls;
+        float2 out[2][FIN_NC];
+        fin_product(stage, wc, l, lane, out);
+#pragma unroll
+        for (int u = 0; u < FIN_NC; ++u) {
+          const int c = c0 + u;
+          if (c >= k) break;
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int rr = lane + 32 * w;
+            if (rr >= nr) break;
+            const float2 v = c < kr ? out[w][u] : make_float2(0.f, 0.f);
+            ur[f * int64_t(n1) * k + r0 + rr + int64_t(n1) * c] = v.x;
+            ui[f * int64_t(n1) * k + r0 + rr + int64_t(n1) * c] = v.y;
+          }
         }
       }
     }
@@ -962,12 +1045,12 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
   const int bf = prec == TP_BF16X3 ? 1 : 0;
   // split planes of the column-major rows x cols matrices (src, ld rows) with
   // K leading dimension ldk
-  auto split = [&](const float* sr, const float* si, int64_t rows, int64_t cols, int conj,
-                   int64_t ldk, float* const* P) {
+  auto split = [&](const float* sr, const float* si, int64_t rows, int64_t cols, int64_t ldk,
+                   float* const* P) {
     {
       KernelScope ks("rsvd_split", st);
       split_planes_kernel<<<grid_for(ldk * cols * h), 256, 0, st>>>(
-          sr, si, rows, cols, rows, rows * cols, h, ldk, ldk * cols, conj, bf, P[0], P[1], P[2],
+          sr, si, rows, cols, rows, rows * cols, h, ldk, ldk * cols, bf, P[0], P[1], P[2],
           P[3]);
     }
     return launch_status("split_planes_kernel");
@@ -993,7 +1076,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
     if (!tc) return hermitian ? gemm(Hr, Hi, n2, n1, br, bi, N, cr, ci)
                               : gemm(Xr, Xi, n1, n2, br, bi, N, cr, ci);
     if (!planes_ready) {
-      int r2 = split(br, bi, K, N, 0, hermitian ? ln : lm, BP);
+      int r2 = split(br, bi, K, N, hermitian ? ln : lm, BP);
       if (r2) return r2;
     }
     planes_ready = false;
@@ -1018,13 +1101,14 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
     // its conjugation) and conj(X_hat) (element (j, i) of X_hat^H at i + ln j)
     {
       KernelScope ks("rsvd_split", st);
+      // lm and ln are at most the next multiple of 32: the tiles cover both
       transpose_split_kernel<<<dim3(unsigned((n1 + 31) / 32), unsigned((lm + 31) / 32),
                                     unsigned(h)),
-                               dim3(32, 8), 0, st>>>(Xr, Xi, n1, n2, lm, bf, XA[0], XA[1], XA[2],
-                                                     XA[3]);
+                               dim3(32, 8), 0, st>>>(Xr, Xi, n1, n2, lm, ln, bf,
+                                                     SplitPlanes{XA[0], XA[1], XA[2], XA[3]},
+                                                     SplitPlanes{XH[0], XH[1], XH[2], XH[3]});
     }
     if ((rc = launch_status("transpose_split_kernel"))) return rc;
-    if ((rc = split(Xr, Xi, n1, n2, 1, ln, XH))) return rc;
   }
   if ((rc = product(false, Or, Oi, l, Yr, Yi))) return rc;     // Y = X_hat Omega
   if ((rc = orth(Yr, Yi, n1))) return rc;
