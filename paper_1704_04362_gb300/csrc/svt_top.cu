@@ -28,7 +28,7 @@
 // and 2 global loads per 16 packed FMAs) and by the certificate's panels, one
 // after the other, half the time each.
 // 41 slices of 144 x 256 (the 144 x 256 x 80 completion), one iteration: 3.5 ms
-// by the warm-started Jacobi and its GEMMs -> 0.61 ms here and 0.14 ms of GEMMs.
+// by the warm-started Jacobi and its GEMMs -> 0.53 ms here and 0.14 ms of GEMMs.
 // From 48 columns on (below, the Jacobi's slices are small and many fit an
 // SM) up to 384, where Q and Y (2 x 2 x 48 KB) still fit the shared memory.
 #include <algorithm>
@@ -57,55 +57,64 @@ struct Tile {   // one row, eight columns
   }
 };
 
+// t += x B[c0 .. c0+7], a row of B in shared memory
+__device__ __forceinline__ void accumulate_one(Tile& t, float xr, float xi, const float* br,
+                                               const float* bi) {
+  const float2 pr = make_float2(xr, xr), pi = make_float2(xi, xi), ni = make_float2(-xi, -xi);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float4 b = reinterpret_cast<const float4*>(br)[h];
+    const float4 d = reinterpret_cast<const float4*>(bi)[h];
+    const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+    const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
+    t.re[2 * h] = __ffma2_rn(pr, b0, t.re[2 * h]);
+    t.re[2 * h + 1] = __ffma2_rn(pr, b1, t.re[2 * h + 1]);
+    t.im[2 * h] = __ffma2_rn(pr, d0, t.im[2 * h]);
+    t.im[2 * h + 1] = __ffma2_rn(pr, d1, t.im[2 * h + 1]);
+    t.re[2 * h] = __ffma2_rn(ni, d0, t.re[2 * h]);
+    t.re[2 * h + 1] = __ffma2_rn(ni, d1, t.re[2 * h + 1]);
+    t.im[2 * h] = __ffma2_rn(pi, b0, t.im[2 * h]);
+    t.im[2 * h + 1] = __ffma2_rn(pi, b1, t.im[2 * h + 1]);
+  }
+}
+
 // t += sum_k A(row, k) B[k][c0 .. c0+7]: A in global memory (column-major,
 // leading dimension lda), B in shared memory (row stride L).  The next eight
-// values of A are loaded before the current ones are used.  (Two rows a thread
-// halve the loads of B but leave too few warps: 70 against 50 thousand cycles
-// for q = 144.)
-__device__ __forceinline__ void accumulate(Tile& t, const float* ar, const float* ai, int64_t lda,
+// values of A are loaded before the current ones are used; whole blocks of
+// eight take no bounds checks and fixed offsets (with two rows of `inner` a
+// warp and the Jacobi's refined reciprocal roots 0.608 -> 0.529 ms a launch for
+// 41 slices of 144 columns).  (Two rows a
+// thread halve the loads of B but leave too few warps: 70 against 50 thousand
+// cycles for q = 144.)
+__device__ __forceinline__ void accumulate(Tile& t, const float* ar, const float* ai, int lda,
                                            int K, const float* Br, const float* Bi, int c0) {
   constexpr int U = 8;
-  float nr[U], ni_[U];
-  auto fetch = [&](int k0) {
+  const int blocks = K / U;
+  const float *br = Br + c0, *bi = Bi + c0;
+  float nr[U], ni[U];
+  auto fetch = [&]() {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const bool in = k0 + u < K;
-      nr[u] = in ? ar[lda * (k0 + u)] : 0.f;
-      ni_[u] = in ? ai[lda * (k0 + u)] : 0.f;
+      nr[u] = *ar;
+      ni[u] = *ai;
+      ar += lda;
+      ai += lda;
     }
   };
-  fetch(0);
-  for (int k0 = 0; k0 < K; k0 += U) {
+  if (blocks > 0) fetch();
+  for (int b = 0; b < blocks; ++b, br += U * L, bi += U * L) {
     float xr[U], xi[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       xr[u] = nr[u];
-      xi[u] = ni_[u];
+      xi[u] = ni[u];
     }
-    fetch(k0 + U);
+    if (b + 1 < blocks) fetch();
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = min(k0 + u, K - 1);
-      const float4* br = reinterpret_cast<const float4*>(Br + k * L + c0);
-      const float4* bi = reinterpret_cast<const float4*>(Bi + k * L + c0);
-      const float2 pr = make_float2(xr[u], xr[u]), pi = make_float2(xi[u], xi[u]);
-      const float2 ni = make_float2(-xi[u], -xi[u]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 b = br[h], d = bi[h];
-        const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
-        const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
-        t.re[2 * h] = __ffma2_rn(pr, b0, t.re[2 * h]);
-        t.re[2 * h + 1] = __ffma2_rn(pr, b1, t.re[2 * h + 1]);
-        t.im[2 * h] = __ffma2_rn(pr, d0, t.im[2 * h]);
-        t.im[2 * h + 1] = __ffma2_rn(pr, d1, t.im[2 * h + 1]);
-        t.re[2 * h] = __ffma2_rn(ni, d0, t.re[2 * h]);
-        t.re[2 * h + 1] = __ffma2_rn(ni, d1, t.re[2 * h + 1]);
-        t.im[2 * h] = __ffma2_rn(pi, b0, t.im[2 * h]);
-        t.im[2 * h + 1] = __ffma2_rn(pi, b1, t.im[2 * h + 1]);
-      }
-    }
+    for (int u = 0; u < U; ++u) accumulate_one(t, xr[u], xi[u], br + u * L, bi + u * L);
   }
+  for (int k = blocks * U; k < K; ++k, ar += lda, ai += lda, br += L, bi += L)
+    accumulate_one(t, *ar, *ai, br, bi);
 }
 
 __device__ __forceinline__ float column(const float2 (&v)[4], int u) {
@@ -124,18 +133,24 @@ struct Shared {
 // of A.
 __device__ void inner(const Shared& s, const float* ar, const float* ai, const float* br,
                       const float* bi, int q, int warp, int lane, int nw) {
-  for (int a = warp; a < L; a += nw) {
-    float sr = 0.f, si = 0.f;
+  // two rows of the result a warp, so that b is read once for both (16 warps;
+  // at least that many run)
+  constexpr int H = L / 2;
+  if (warp >= H) return;
+  float2 sr = make_float2(0.f, 0.f), si = sr;
 #pragma unroll 4
-    for (int k = 0; k < q; ++k) {
-      const float xr = ar[k * L + a], xi = ai[k * L + a];
-      const float yr = br[k * L + lane], yi = bi[k * L + lane];
-      sr = fmaf(xr, yr, fmaf(xi, yi, sr));
-      si = fmaf(xr, yi, fmaf(-xi, yr, si));
-    }
-    s.Sr[a * LS + lane] = sr;
-    s.Si[a * LS + lane] = si;
+  for (int k = 0; k < q; ++k) {
+    const float2 xr = make_float2(ar[k * L + warp], ar[k * L + warp + H]);
+    const float2 xi = make_float2(ai[k * L + warp], ai[k * L + warp + H]);
+    const float yr = br[k * L + lane], yi = bi[k * L + lane];
+    const float2 pr = make_float2(yr, yr), pi = make_float2(yi, yi), nr = make_float2(-yr, -yr);
+    sr = __ffma2_rn(xr, pr, __ffma2_rn(xi, pi, sr));
+    si = __ffma2_rn(xr, pi, __ffma2_rn(xi, nr, si));
   }
+  s.Sr[warp * LS + lane] = sr.x;
+  s.Si[warp * LS + lane] = si.x;
+  s.Sr[(warp + H) * LS + lane] = sr.y;
+  s.Si[(warp + H) * LS + lane] = si.y;
 }
 
 // dst = src M (q x L, L x L), M(b, c) at mr[b * LS + col], col = order[c] or c.
@@ -230,6 +245,12 @@ __device__ void fill_pairs(uchar2* pairs, int tid, int nt) {
   }
 }
 
+// 1 / sqrt(x), the hardware's value after one Newton-Raphson step
+__device__ __forceinline__ float rsqrt_refined(float x) {
+  const float y = rsqrtf(x);
+  return y * fmaf(-0.5f * x, y * y, 1.5f);
+}
+
 // Two-sided Jacobi of the Hermitian S: S <- Z^H S Z, Z accumulated, with its
 // entries off the diagonal below 5e-8 of the largest diagonal one wherever a
 // pair could hold an eigenvalue above t2 (the vectors below the threshold need
@@ -262,11 +283,15 @@ __device__ void small_jacobi(const Shared& s, float t2, int tid, int nt, const u
         // rotation by (c, s e^{i phi}) with gamma = |gamma| e^{i phi}
         float c = 1.f, sr = 0.f, si = 0.f;
         if (g2 > small && al + be > 0.98f * t2) {
-          const float g = sqrtf(g2), z = (be - al) / (2.f * g);
-          const float t = copysignf(1.f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
-          c = 1.f / sqrtf(fmaf(t, t, 1.f));
-          sr = c * t * gr / g;
-          si = c * t * gi / g;
+          // refined reciprocal square roots: the step's chain is half as long as
+          // with the rounded roots and divisions (c and e^{i phi} are unit to
+          // rounding whatever the error of t)
+          const float ig = rsqrt_refined(g2), z = 0.5f * (be - al) * ig;
+          const float w = fmaf(z, z, 1.f);
+          const float t = __fdividef(copysignf(1.f, z), fabsf(z) + w * rsqrt_refined(w));
+          c = rsqrt_refined(fmaf(t, t, 1.f));
+          sr = c * t * (gr * ig);
+          si = c * t * (gi * ig);
           turn = true;
         }
         rot[tid] = make_float4(c, sr, si, 0.f);
