@@ -112,20 +112,23 @@ __global__ void horizontal_partial_kernel(const float* __restrict__ X, int64_t n
 
 // out[i] = sum over the G chunk partials of row i (partial[g * n1 + i]; for the
 // lateral norms row j has the n3 partials of its columns): a block takes 4 rows
-// (a sector), its 64 thread groups each sum a contiguous part of the chunks
-// (loads batched, adds in chunk order), then the parts are added in order, 8
-// and 8; the same partition for a given G, so every norm is deterministic.
+// (a sector), its SEG thread groups each sum a contiguous part of the chunks
+// (loads batched, adds in chunk order), then the parts are added in order,
+// eight at a time and those; the same partition for a given G, so every norm is
+// deterministic.
 // Bound by the float64 adds (two a cycle and SM), so the rows are spread over
 // as many blocks as possible: 192 rows of 4864 partials and 1140 of 168, one
-// thread a row 0.261 ms together, 32 rows a block 0.072 -> 0.038.
-constexpr int NR_ROWS = 4, NR_SEG = 64;
+// thread a row 0.261 ms together, 32 rows a block 0.072, 64 groups for both
+// 0.038 -> 0.026 with 256 where there are more than 1024 partials.
+constexpr int NR_ROWS = 4;
 
-__global__ void __launch_bounds__(NR_ROWS * NR_SEG)
+template <int SEG>
+__global__ void __launch_bounds__(NR_ROWS * SEG)
     norms_reduce_kernel(const double* __restrict__ partial, int64_t n1, int64_t G,
                         double* __restrict__ out) {
-  __shared__ double part[NR_SEG][NR_ROWS], eighth[8][NR_ROWS];
+  __shared__ double part[SEG][NR_ROWS], eights[SEG / 8][NR_ROWS];
   const int lr = threadIdx.x % NR_ROWS, seg = threadIdx.x / NR_ROWS;
-  const int64_t S = (G + NR_SEG - 1) / NR_SEG;
+  const int64_t S = (G + SEG - 1) / SEG;
   for (int64_t r0 = int64_t(blockIdx.x) * NR_ROWS; r0 < n1; r0 += int64_t(gridDim.x) * NR_ROWS) {
     const int64_t i = r0 + lr;
     double a = 0.0;
@@ -136,17 +139,17 @@ __global__ void __launch_bounds__(NR_ROWS * NR_SEG)
     }
     part[seg][lr] = a;
     __syncthreads();
-    if (seg < 8) {
+    if (seg < SEG / 8) {
       double t = 0.0;
 #pragma unroll
       for (int k = 0; k < 8; ++k) t += part[8 * seg + k][lr];
-      eighth[seg][lr] = t;
+      eights[seg][lr] = t;
     }
     __syncthreads();
     if (seg == 0 && i < n1) {
       double t = 0.0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) t += eighth[k][lr];
+      for (int k = 0; k < SEG / 8; ++k) t += eights[k][lr];
       out[i] = t;
     }
   }
@@ -162,7 +165,10 @@ void launch_norms_reduce(const double* partial, int64_t n1, int64_t G, double* o
     return;
   }
   const int64_t rb = std::min<int64_t>((n1 + NR_ROWS - 1) / NR_ROWS, int64_t(sm_count()) * 8);
-  norms_reduce_kernel<<<unsigned(rb), NR_ROWS * NR_SEG, 0, st>>>(partial, n1, G, out);
+  if (G <= 1024)
+    norms_reduce_kernel<64><<<unsigned(rb), NR_ROWS * 64, 0, st>>>(partial, n1, G, out);
+  else
+    norms_reduce_kernel<256><<<unsigned(rb), NR_ROWS * 256, 0, st>>>(partial, n1, G, out);
 }
 
 int64_t horizontal_chunks(int64_t n1, int64_t ncols) {
