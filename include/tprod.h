@@ -219,9 +219,12 @@ int tsvd_randomized(const float* X, int64_t n1, int64_t n2, int64_t n3,
  * Z = C * C^dagger * A (n1 x n2 x n3 output), computed per half-spectrum
  * slice as P_k A_hat_k with P_k the projector onto range(C_hat_k), whose
  * basis is the left singular vectors of C_hat_k (float64 Jacobi) above
- * MATLAB's pinv cut-off max(n1, c') eps(s_max).
+ * MATLAB's pinv cut-off max(n1, c') eps(s_max) or, where up to 96 picked
+ * slices (c' <= n1) are clearly of full rank in every frequency, a Householder
+ * QR of C_hat_k.
  *   idx_out / count_out: as tprod_sampled.
- * Reads the pick count back to the host once (synchronises `stream`).
+ * Reads the pick count, and with the QR its rank check, back to the host
+ * (synchronises `stream`).
  * Limits: min(n1, n2) <= 512, n2 <= 4096, n3 <= 512.                        */
 int tcx(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint64_t seed,
         int prob_mode, const double* p_given, float* Z, int32_t* idx_out, int64_t* count_out,
@@ -300,11 +303,13 @@ int cur_tnn(const float* X, const uint8_t* mask, int64_t n1, int64_t n2, int64_t
  *            previous outputs resumes it)
  *   mu    device float64 scalar, read and updated in place
  * Paper constants: mu0 = 1e-3, rho = 1.1, mu_max = 1e10.  The slice SVT
- * takes V from a float32 one-sided Jacobi (warm-started from the previous
- * iteration's V within a call) and the singular values as Rayleigh quotients
- * ||W v_j|| / ||v_j||.  Resuming from the returned state agrees with one
- * longer call to float32 rounding (the Jacobi's starting rotations are not
- * part of the state).  Limits as tsvd.                                      */
+ * takes the right singular vectors above the threshold from 32 vectors kept
+ * from iteration to iteration within a call (48 <= min(n1, n2) <= 384;
+ * certified to be complete), else and where that does not certify all of V
+ * from a float32 one-sided Jacobi (warm-started likewise), and the singular
+ * values as Rayleigh quotients ||W v_j|| / ||v_j||.  Resuming from the
+ * returned state agrees with one longer call to float32 rounding (the vectors
+ * that an iteration starts from are not part of the state).  Limits as tsvd. */
 int tcomplete_svt(const float* X, const uint8_t* mask,
                   int64_t n1, int64_t n2, int64_t n3, int iters,
                   double rho, double mu_max,

@@ -2,7 +2,9 @@
 // (Section 2, "Operators": fft(X,[],3) / ifft(X,[],3); Algorithm 1 steps 2-3
 // and the final inverse).
 //
-// Both directions are small dense contractions per tube.  The t <-> n3 - t
+// The transforms of lengths that neither rfft_reg.cu (registers) nor fft.cu
+// (primes up to 13) takes, and the choice among the three.  Both directions
+// are small dense contractions per tube.  The t <-> n3 - t
 // symmetry halves them: with e_t = x_t + x_{n3-t} and o_t = x_t - x_{n3-t}
 // (t = 1 .. n3/2; e_0 = x_0 and, for even n3, e_{n3/2} = x_{n3/2}, o = 0 there),
 //     Re X_k = sum_{t <= n3/2} e_t cos(2 pi k t / n3),

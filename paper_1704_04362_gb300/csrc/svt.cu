@@ -8,7 +8,9 @@
 //   E = (X_obs - L - Y/mu) off the mask, 0 on it
 //   Y = Y + mu (L + E - X_obs)                    (admm_post_kernel)
 //   mu = min(rho mu, mu_max)                      (admm_mu_kernel)
-// X_obs is X where the mask is set and 0 elsewhere.  The slice SVT takes the
+// X_obs is X where the mask is set and 0 elsewhere.  Slices of 48 to 384 columns
+// take the few vectors above the threshold from svt_top.cu; for the others, and
+// where that does not certify them, the slice SVT takes the
 // right singular vectors V from the float32 one-sided Jacobi of svd.cu on a
 // copy of M_hat_k (or its conjugate transpose when n1 < n2), warm-started
 // from the previous iteration's V (the ADMM iterate moves little between

@@ -63,7 +63,9 @@ inline size_t ws_bytes(size_t count, size_t elem) { return (count * elem + 255) 
 int acquire_workspace(const tp_opts* opts, size_t need, Arena* out, size_t least = 0,
                       bool* lean = nullptr);
 
-__host__ __device__ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+__host__ __device__ inline bool aligned16(const void* p) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+}
 inline int64_t half_len(int64_t n3) { return n3 / 2 + 1; }
 
 // ---------------------------------------------------------------- kernels
