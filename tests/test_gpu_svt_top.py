@@ -93,3 +93,30 @@ def test_zero_and_scaled_data(scale):
     Lr, _, _, _ = completion_ref.tcomplete_svt(X.astype(np.float64), mask, 2, mu0=mu0)
     assert rel_fro(L, Lr) <= 2 * TOL_FP32 if scale else not np.any(L)
     assert not np.any(E)
+
+
+@pytest.mark.parametrize("short", [0, 256, 1 << 30])
+def test_a_workspace_without_the_kept_vectors(short, monkeypatch):
+    """256 bytes fewer than asked for: every slice takes the Jacobi; far too
+    few are refused."""
+    from paper_1704_04362_gb300 import binding
+    X = synth.lowrank_np(70, 64, 6, 4, seed=3, noise=0.02)
+    mask = np.asfortranarray((np.random.default_rng(1).random(X.shape) < 0.6).astype(np.uint8))
+    mu0 = threshold(X, 0.3)
+    plain = binding._opts
+
+    def less(op, dims, *args, **kw):
+        import ctypes
+        o = plain(op, dims, *args, **kw)
+        d = (ctypes.c_int64 * len(dims))(*dims)
+        need = binding.lib().tp_workspace_query(op, ctypes.addressof(d), len(dims), ctypes.byref(o))
+        o.workspace_bytes = max(need - short, 0)
+        return o
+
+    monkeypatch.setattr(binding, "_opts", less)
+    if short > 256:
+        with pytest.raises(Exception):
+            run(X, mask, 4, mu0)
+        return
+    compare(X, mask, 4, mu0)
+    compare(X, mask, 4, mu0, batch=True)
