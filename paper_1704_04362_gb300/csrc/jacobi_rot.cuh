@@ -7,6 +7,18 @@
 namespace tp {
 namespace jrot {
 
+// gamma and beta - alpha times a power of two that brings |gamma| near 1, and
+// the scaled |gamma|: where its square nears or leaves the normal range (null
+// columns of a rank-deficient slice), e^{-i phi} from the root of that square
+// would not be of unit length and V would lose its orthonormality.  Out of line:
+// the common case pays a compare.
+static __device__ __noinline__ float4 rotation_tiny(float gr, float gi, float d) {
+  int e;
+  frexpf(fmaxf(fabsf(gr), fabsf(gi)), &e);
+  const float a = ldexpf(gr, -e), b = ldexpf(gi, -e);
+  return make_float4(a, b, ldexpf(d, -e), sqrtf(a * a + b * b));
+}
+
 // Jacobi rotation of a pair from its two diagonal terms alpha, beta (the
 // squared column norms of a one-sided sweep, or the diagonal entries of a
 // Hermitian matrix) and its off-diagonal term gamma = gr + i gi, g2 =
@@ -17,25 +29,22 @@ namespace jrot {
 // and ||b'||^2 = beta + tg.
 __device__ __forceinline__ void rotation(float alpha, float beta, float gr, float gi, float g2,
                                          float& cs, float& sn, float& er, float& ei, float& tg) {
-  float g = sqrtf(g2);
-  er = gr / g;
-  ei = -gi / g;
+  float g = sqrtf(g2), d = beta - alpha, back = 1.f;
   if (g2 < 1e-30f) {
-    // g2 nears or leaves the normal range (null columns of a rank-deficient
-    // slice) and its root with it: gamma scaled by a power of two first, or
-    // e^{-i phi} is not of unit length and V loses its orthonormality
-    int e;
-    frexpf(fmaxf(fabsf(gr), fabsf(gi)), &e);
-    const float a = ldexpf(gr, -e), b = ldexpf(gi, -e), gs = sqrtf(a * a + b * b);
-    er = a / gs;
-    ei = -b / gs;
-    g = ldexpf(gs, e);
+    const float4 r = rotation_tiny(gr, gi, d);
+    back = r.x != 0.f ? gr / r.x : gi / r.y;
+    gr = r.x;
+    gi = r.y;
+    d = r.z;
+    g = r.w;
   }
-  const float zeta = (beta - alpha) / (2.f * g);
+  const float zeta = d / (2.f * g);
   const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
   cs = 1.f / sqrtf(1.f + t * t);
   sn = cs * t;
-  tg = t * g;
+  er = gr / g;
+  ei = -gi / g;
+  tg = t * g * back;
 }
 __device__ __forceinline__ void rotation(float alpha, float beta, float gr, float gi, float g2,
                                          float& cs, float& sn, float& er, float& ei) {
@@ -63,11 +72,12 @@ __device__ __forceinline__ void rotation(double alpha, double beta, double gr, d
   const float af = float(alpha * sc), bf = float(beta * sc), g2f = float(g2 * sc * sc);
   // outside float's range after scaling (|gamma| far below the norms, or norms
   // kept through cancellation far below |gamma|): all in float64
-  if (!(g2f > 1e-30f && g2f < 1e30f) || g2 < 1e-290) {
+  const bool tiny = __double2hiint(g2) < 0x03c00000;   // g2 < 1e-290
+  if (tiny || !(g2f > 1e-30f && g2f < 1e30f)) {
     double g = sqrt(g2);
     er = gr / g;
     ei = -gi / g;
-    if (g2 < 1e-290) {   // as in float32: gamma scaled before its square
+    if (tiny) {   // as in float32: gamma scaled before its square
       frexp(fmax(fabs(gr), fabs(gi)), &e);
       const double a = ldexp(gr, -e), b = ldexp(gi, -e), gs = sqrt(a * a + b * b);
       er = a / gs;
