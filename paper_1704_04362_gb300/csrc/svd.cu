@@ -1080,12 +1080,18 @@ int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T*
                           int32_t* status, int flags, cudaStream_t st,
                           const int* skip = nullptr) {
   if (batch <= 0 || q <= 0) return TP_OK;
-  const size_t smem = jacobi_cluster_smem<T>(p, q), ring = jacobi_ring_smem<T>(p, q);
+  // The ring where it is the faster one: float32 pairs that fit the registers
+  // (120 x 100 x 6: 1.91 -> 1.13 ms), or enough columns that a round's rotations
+  // outweigh pushing its columns (256 x 200: float32 5.05 -> 3.95, float64 15.3
+  // and 15.4 ms; 256 x 150 float64 16.9 -> 13.3).  256 x 64 through L2 against the
+  // ring: float32 1.41 / 1.52, float64 1.99 / 2.32 ms.
+  constexpr bool f32 = sizeof(T) == 4;
+  const bool faster = (f32 && std::max(p, q) <= 128) || q >= 96;
+  const size_t smem = jacobi_cluster_smem<T>(p, q), ring = faster ? jacobi_ring_smem<T>(p, q) : 0;
   const unsigned grid = unsigned(batch) * JPC;
   {
     KernelScope ks(sizeof(T) == 4 ? "jacobi_f32" : "jacobi_svd", st);
     if (ring) {
-      constexpr bool f32 = sizeof(T) == 4;
       auto kernel = f32 && std::max(p, q) <= 64    ? jacobi_ring_kernel<T, f32 ? 2 : 0>
                     : f32 && std::max(p, q) <= 128 ? jacobi_ring_kernel<T, f32 ? 4 : 0>
                                                    : jacobi_ring_kernel<T, 0>;
