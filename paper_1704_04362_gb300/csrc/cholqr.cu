@@ -1,0 +1,249 @@
+// orth() of tall slices in float64: CholeskyQR2 of a batch of slices (p x l,
+// l <= 96, planar float32, column-major) with float64 Gram matrices, Cholesky
+// factors and solves; only Y itself is rounded to float32, once a pass.
+//
+//   G = Y^H Y,  G = R^H R,  Y <- Y R^{-1},   twice
+// (Fukaya, Nakatsukasa, Yanagisawa and Yamamoto 2014); a Cholesky breakdown is
+// retried once with the diagonal shifted by 11 (p l + l (l + 1)) u ||Y||_F^2,
+// followed by two plain passes (shifted CholeskyQR3).
+//
+// Bound by the float64 pipe (two lanes a cycle and SM): a Gram entry is six
+// operations a row, a solve six per entry of R and row.  So the Gram entries are
+// spread over blocks by pairs of columns and the solves by rows, and every
+// operand is converted to float64 once per block instead of once per use.  Every
+// entry's sum runs over the rows (the solve's over the columns) in order, so
+// the split changes no result.  33 slices of 1024 x 50: one block per slice
+// 14.5 ms -> 3.2 ms.
+#include "householder.cuh"
+
+namespace tp {
+namespace {
+
+constexpr int GRAM_THREADS = 128;   // column pairs a block
+constexpr int GRAM_ROWS = 32;       // rows staged at once
+constexpr int FACTOR_THREADS = 256;
+
+// State of a slice between the launches of a pass.
+struct Progress {
+  int passes;    // passes left
+  int shifted;   // the next pass adds the shift
+  int solve;     // this pass has a factor
+};
+
+struct CholArgs {
+  float *yr, *yi;          // element (r, c) of slice f at f*sY + r + p*c
+  int64_t sY;
+  int p, lfull;
+  const int32_t* lcols;    // per-slice column counts or null
+  double2* G;              // [slice][l][l], row-major: the Gram matrix, then R
+  Progress* state;
+  int32_t* status;
+  int* weak;               // see householder.cuh
+  int first;               // pass 0: every slice takes part
+};
+
+__device__ __forceinline__ int columns_of(const CholArgs& g, int f) {
+  return g.lcols ? min(max(int(g.lcols[f]), 1), g.lfull) : g.lfull;
+}
+
+// Upper triangle of G, one pair of columns a thread; the block's rows arrive in
+// chunks of GRAM_ROWS as float64 in shared memory (row pitch odd, so that
+// neither the writes along a column nor the reads along a row conflict).
+__global__ void __launch_bounds__(GRAM_THREADS) cholqr_gram_kernel(const CholArgs g) {
+  extern __shared__ __align__(16) double2 chol_sm[];
+  const int f = blockIdx.y, l = columns_of(g, f), p = g.p, pitch = l | 1;
+  if (!g.first && g.state[f].passes <= 0) return;
+  const int npairs = l * (l + 1) / 2, e0 = int(blockIdx.x) * GRAM_THREADS;
+  if (e0 >= npairs) return;
+  const float* yr = g.yr + int64_t(f) * g.sY;
+  const float* yi = g.yi + int64_t(f) * g.sY;
+  // e -> (a, b), a <= b, row-major upper triangle
+  int a = 0, rem = min(e0 + int(threadIdx.x), npairs - 1);
+  while (rem >= l - a) rem -= l - a, ++a;
+  const int b = a + rem;
+  double sr = 0.0, si = 0.0;
+  for (int r0 = 0; r0 < p; r0 += GRAM_ROWS) {
+    const int nr = min(GRAM_ROWS, p - r0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < GRAM_ROWS * l; e += GRAM_THREADS) {
+      const int r = e % GRAM_ROWS, c = e / GRAM_ROWS;
+      if (r >= nr) continue;
+      const int64_t o = r0 + r + int64_t(p) * c;
+      chol_sm[r * pitch + c] = make_double2(double(yr[o]), double(yi[o]));
+    }
+    __syncthreads();
+    for (int r = 0; r < nr; ++r) {
+      const double2 x = chol_sm[r * pitch + a], y = chol_sm[r * pitch + b];
+      const double ar = x.x, ai = x.y, br = y.x, bi = y.y;
+      sr += ar * br + ai * bi;   // products of float32 values: exact
+      si += ar * bi - ai * br;
+    }
+  }
+  if (e0 + int(threadIdx.x) < npairs)
+    g.G[(int64_t(f) * g.lfull + a) * g.lfull + b] = make_double2(sr, si);
+}
+
+// R of every slice whose Gram matrix was formed (upper triangle of G in place),
+// one block a slice; sets what the slice does next.
+__global__ void __launch_bounds__(FACTOR_THREADS) cholqr_factor_kernel(const CholArgs g) {
+  extern __shared__ __align__(16) double2 chol_sm[];   // l x l, row-major
+  __shared__ int bad;
+  const int f = blockIdx.x, l = columns_of(g, f), tid = threadIdx.x;
+  Progress s = g.first ? Progress{2, 0, 0} : g.state[f];
+  if (s.passes <= 0) {
+    if (tid == 0) g.state[f].solve = 0;
+    return;
+  }
+  double2* Gf = g.G + int64_t(f) * g.lfull * g.lfull;
+  for (int e = tid; e < l * l; e += FACTOR_THREADS) {
+    const int a = e / l, b = e - a * l;
+    if (a <= b) chol_sm[e] = Gf[a * g.lfull + b];
+  }
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  if (s.shifted) {
+    if (tid == 0) {
+      double tr = 0.0;
+      for (int j = 0; j < l; ++j) tr += chol_sm[j * l + j].x;
+      const double sh = 11.0 * (double(g.p) * l + double(l) * (l + 1)) * 1.1102230246251565e-16 * tr;
+      for (int j = 0; j < l; ++j) chol_sm[j * l + j].x += sh;
+    }
+    __syncthreads();
+  }
+  // row i of R, then its share of every entry right of and below it
+  const int lane = tid & 31, warp = tid >> 5;
+  for (int i = 0; i < l; ++i) {
+    const double d = chol_sm[i * l + i].x;
+    if (!(d > 0.0) || !isfinite(d)) {   // the same for every thread
+      if (tid == 0) bad = 1;
+      break;
+    }
+    const double dii = sqrt(d);
+    __syncthreads();
+    for (int k = i + tid; k < l; k += FACTOR_THREADS) {
+      const double2 v = chol_sm[i * l + k];
+      chol_sm[i * l + k] = k == i ? make_double2(dii, 0.0) : make_double2(v.x / dii, v.y / dii);
+    }
+    __syncthreads();
+    for (int j = i + 1 + warp; j < l; j += FACTOR_THREADS / 32) {
+      const double2 x = chol_sm[i * l + j];
+      for (int k = j + lane; k < l; k += 32) {   // subtract conj(R_ij) R_ik
+        const double2 y = chol_sm[i * l + k], v = chol_sm[j * l + k];
+        const double ar = x.x, ai = x.y, br = y.x, bi = y.y;
+        double sr = v.x, si = v.y;
+        sr -= ar * br + ai * bi;
+        si -= ar * bi - ai * br;
+        chol_sm[j * l + k] = make_double2(sr, si);
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  const bool ok = bad == 0;
+  if (ok)
+    for (int e = tid; e < l * l; e += FACTOR_THREADS) {
+      const int a = e / l, b = e - a * l;
+      if (a <= b) Gf[a * g.lfull + b] = chol_sm[e];
+    }
+  if (tid != 0) return;
+  if (g.first && g.weak) {
+    double lo = INFINITY, hi = 0.0;
+    for (int j = 0; j < l && ok; ++j) {
+      lo = fmin(lo, chol_sm[j * l + j].x);
+      hi = fmax(hi, chol_sm[j * l + j].x);
+    }
+    if (!ok || !(lo > double(HQR_WEAK) * hi)) atomicOr(g.weak, 1);
+  }
+  s.solve = ok;
+  if (ok) {
+    s.shifted = 0;
+    --s.passes;
+  } else if (s.shifted) {   // left as it is
+    s.passes = 0;
+    if (g.status) atomicOr(g.status, TP_DEV_BREAKDOWN);
+  } else {
+    s.shifted = 1;   // this pass again with a shift, then two plain ones
+    s.passes = 3;
+  }
+  g.state[f] = s;
+}
+
+// Y <- Y R^{-1}, a thread a row (x R = y by forward substitution); in pass 0
+// the columns past the slice's count are set to zero.
+__global__ void cholqr_solve_kernel(const CholArgs g) {
+  extern __shared__ __align__(16) double2 chol_sm[];
+  const int f = blockIdx.y, l = columns_of(g, f), p = g.p, T = blockDim.x, tid = threadIdx.x;
+  const int r = int(blockIdx.x) * T + tid;
+  float* yr = g.yr + int64_t(f) * g.sY + r;
+  float* yi = g.yi + int64_t(f) * g.sY + r;
+  if (g.first && r < p)
+    for (int c = l; c < g.lfull; ++c) yr[int64_t(p) * c] = yi[int64_t(p) * c] = 0.f;
+  if (!g.state[f].solve) return;
+  double2* R = chol_sm;             // l x l, row-major
+  double2* x = chol_sm + l * l;     // x[i * T + tid]
+  const double2* Gf = g.G + int64_t(f) * g.lfull * g.lfull;
+  for (int e = tid; e < l * l; e += T) {
+    const int a = e / l, b = e - a * l;
+    if (a <= b) R[e] = Gf[a * g.lfull + b];
+  }
+  __syncthreads();
+  if (r >= p) return;
+  for (int j = 0; j < l; ++j) {
+    double sr = yr[int64_t(p) * j], si = yi[int64_t(p) * j];
+    for (int i = 0; i < j; ++i) {
+      const double2 v = x[i * T + tid], w = R[i * l + j];
+      const double xr = v.x, xi = v.y, ar = w.x, ai = w.y;
+      sr -= xr * ar - xi * ai;
+      si -= xr * ai + xi * ar;
+    }
+    const double d = R[j * l + j].x;
+    const float qr = float(sr / d), qi = float(si / d);
+    yr[int64_t(p) * j] = qr;
+    yi[int64_t(p) * j] = qi;
+    x[j * T + tid] = make_double2(double(qr), double(qi));
+  }
+}
+
+size_t solve_smem(int l, int T) { return (size_t(l) * l + size_t(l) * T) * sizeof(double2); }
+
+}  // namespace
+
+size_t cholqr_scratch(int64_t l, int64_t batch) {
+  return ws_bytes(size_t(l) * l * batch, sizeof(double2)) + ws_bytes(size_t(batch), sizeof(Progress));
+}
+
+int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak) {
+  if (l < 1 || l > HQR_MAX_L || rows < l || rows > 0x7fffffff || batch > 65535) {
+    set_error("cholqr: needs l <= rows, l <= %d and at most 65535 slices", HQR_MAX_L);
+    return TP_EUNSUPPORTED;
+  }
+  if (batch <= 0) return TP_OK;
+  Arena ws;
+  ws.base = static_cast<char*>(scratch);
+  CholArgs g{yr, yi, rows * l, int(rows), l, lcols, nullptr, nullptr, status, weak, 1};
+  g.G = ws.take<double2>(size_t(l) * l * batch);
+  g.state = ws.take<Progress>(size_t(batch));
+  const size_t gram_smem = size_t(GRAM_ROWS) * (l | 1) * sizeof(double2);
+  const size_t factor_smem = size_t(l) * l * sizeof(double2);
+  // rows a block: two blocks an SM where they fit
+  int T = 128;
+  while (T > 32 && solve_smem(l, T) > size_t(100) * 1024) T /= 2;
+  TP_SET_SMEM(cholqr_gram_kernel, gram_smem);
+  TP_SET_SMEM(cholqr_factor_kernel, factor_smem);
+  TP_SET_SMEM(cholqr_solve_kernel, solve_smem(l, T));
+  const unsigned pairs = unsigned((l * (l + 1) / 2 + GRAM_THREADS - 1) / GRAM_THREADS);
+  const unsigned blocks = unsigned((rows + T - 1) / T), slices = unsigned(batch);
+  // four passes at most: the breakdown, its shifted repeat and two plain ones
+  for (int it = 0; it < 4; ++it) {
+    g.first = it == 0;
+    KernelScope ks("cholqr", st);
+    cholqr_gram_kernel<<<dim3(pairs, slices), GRAM_THREADS, gram_smem, st>>>(g);
+    cholqr_factor_kernel<<<slices, FACTOR_THREADS, factor_smem, st>>>(g);
+    cholqr_solve_kernel<<<dim3(blocks, slices), T, solve_smem(l, T), st>>>(g);
+    note_launches(2);
+  }
+  return launch_status("cholqr");
+}
+
+}  // namespace tp

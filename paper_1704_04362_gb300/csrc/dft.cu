@@ -512,6 +512,18 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
   return rc ? rc : run(c);
 }
 
+// The plain forward transform with every frequency's samples summed in order
+// (tubes of 17 to 256 samples that are no power of two up to 128), for callers
+// whose results hang on the rounding of its sums; else launch_rdft.
+int launch_rdft_in_order(const DftGather& g, cudaStream_t st) {
+  if (g.n3 <= 16 || g.n3 > 256 || rfft_reg_supported(g.n3)) return launch_rdft(g, st);
+  if (g.rows == 0 || g.cols == 0) return TP_OK;
+  DftArgs p{};
+  p.g = g;
+  p.n3 = int(g.n3);
+  return launch_product<false>(p, g.rows * g.cols, "rdft", st);
+}
+
 int launch_irdft(const float* in_re, const float* in_im, int64_t rows, int64_t in_slice,
                  int64_t n3, float* out, cudaStream_t st) {
   if (n3 < 1 || (n3 > 512 && !fft_supported(n3))) {

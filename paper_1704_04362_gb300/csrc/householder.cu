@@ -580,6 +580,174 @@ int hqr_dispatch(const HqrParams& g, int p, int64_t blocks, cudaStream_t st) {
   return hqr_launch<4, 16, 6, MODE>(g, blocks, st);
 }
 
+// ---------------------------------------------------------------- in shared memory
+//
+// The same QR of a slice of at most 256 rows held in shared memory, a step's
+// reflector in registers (lane r % 32 holds rows r) and a warp per column.  It
+// is a few percent slower than the registers' form above and rounds in another
+// order.  The sketch without power iterations takes it: there the trailing
+// singular values are set by the rounding of the core's Gram matrix (rsvd.cu),
+// so that another order of the sums here moves them by more than rounding.
+constexpr int HQS_THREADS = 256;
+constexpr int HQS_WARPS = HQS_THREADS / 32;
+
+// Reflector of column a (rows j .. p-1), one warp: rows j+1.. become v,
+// row j becomes beta; returns tau (0 when the column is already beta e_j with
+// beta real).
+__device__ float2 hqs_reflector(float2* a, int j, int p, int lane) {
+  const float2 al = a[j];
+  float s = 0.f;
+  for (int r = j + 1 + lane; r < p; r += 32) {
+    const float2 x = a[r];
+    s = fmaf(x.x, x.x, fmaf(x.y, x.y, s));
+  }
+  s = hqr_sum(s);
+  if (s == 0.f && al.y == 0.f) return make_float2(0.f, 0.f);
+  const float nrm = sqrtf(fmaf(al.x, al.x, fmaf(al.y, al.y, s)));
+  const float beta = al.x >= 0.f ? -nrm : nrm;
+  // v = x / (alpha - beta); |alpha - beta| >= nrm > 0 by the sign of beta
+  const float dr = al.x - beta, di = al.y;
+  const float den = fmaf(dr, dr, di * di);
+  const float sr = dr / den, si = -di / den;
+  for (int r = j + 1 + lane; r < p; r += 32) {
+    const float2 x = a[r];
+    a[r] = make_float2(x.x * sr - x.y * si, x.x * si + x.y * sr);
+  }
+  __syncwarp();
+  if (lane == 0) a[j] = make_float2(beta, 0.f);
+  return make_float2((beta - al.x) / beta, -al.y / beta);
+}
+
+// v_j of column a into registers: row r = lane + 32 t, 1 at row j, 0 above.
+template <int RPL>
+__device__ __forceinline__ void hqs_load_v(const float2* a, int j, int p, int lane,
+                                           float2 (&v)[RPL]) {
+#pragma unroll
+  for (int t = 0; t < RPL; ++t) {
+    const int r = lane + 32 * t;
+    v[t] = (r <= j || r >= p) ? make_float2(r == j ? 1.f : 0.f, 0.f) : a[r];
+  }
+}
+
+// c <- c - f v (v^H c) on rows j .. p-1 (f = conj(tau) applies H^H, f = tau H)
+template <int RPL>
+__device__ __forceinline__ void hqs_apply(const float2 (&v)[RPL], float2* c, int j, int p, float2 f,
+                                          int lane) {
+  float2 x[RPL];
+  float dr = 0.f, di = 0.f;
+#pragma unroll
+  for (int t = 0; t < RPL; ++t) {
+    const int r = lane + 32 * t;
+    x[t] = (r >= j && r < p) ? c[r] : make_float2(0.f, 0.f);
+    dr = fmaf(v[t].x, x[t].x, fmaf(v[t].y, x[t].y, dr));    // Re(conj(v) x)
+    di = fmaf(v[t].x, x[t].y, fmaf(-v[t].y, x[t].x, di));   // Im(conj(v) x)
+  }
+  hqr_sum2(dr, di, lane);
+  const float gr = f.x * dr - f.y * di, gi = f.x * di + f.y * dr;
+#pragma unroll
+  for (int t = 0; t < RPL; ++t) {
+    const int r = lane + 32 * t;
+    if (r >= j && r < p)
+      c[r] = make_float2(x[t].x - (v[t].x * gr - v[t].y * gi),
+                         x[t].y - (v[t].x * gi + v[t].y * gr));
+  }
+}
+
+// Column k of Q from its reflector (stored in place): H_k e_k restricted to
+// rows k.. -- 1 - tau at row k, -tau v below -- and zeros above.
+__device__ __forceinline__ void hqs_materialize(float2* a, int k, int p, float2 tau, int lane) {
+  for (int r = lane; r < p; r += 32) {
+    float2 y;
+    if (r < k) {
+      y = make_float2(0.f, 0.f);
+    } else if (r == k) {
+      y = make_float2(1.f - tau.x, -tau.y);
+    } else {
+      const float2 v = a[r];
+      y = make_float2(-(tau.x * v.x - tau.y * v.y), -(tau.x * v.y + tau.y * v.x));
+    }
+    a[r] = y;
+  }
+}
+
+// One CTA per slice; RPL rows per lane (p <= 32 RPL).
+template <int RPL>
+__global__ void __launch_bounds__(HQS_THREADS) householder_shared_kernel(float* y_re, float* y_im,
+                                                                         int64_t sY, int p,
+                                                                         int lfull,
+                                                                         const int32_t* lcols) {
+  extern __shared__ __align__(16) float2 hqs_a[];   // Y, then Q: p x l column-major
+  __shared__ float2 tau_s[HQR_MAX_L];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int l = lcols ? min(max(int(lcols[blockIdx.x]), 1), lfull) : lfull;
+  float* yr = y_re + int64_t(blockIdx.x) * sY;
+  float* yi = y_im + int64_t(blockIdx.x) * sY;
+  float2* A = hqs_a;
+  for (int e = threadIdx.x; e < p * l; e += HQS_THREADS) A[e] = make_float2(yr[e], yi[e]);
+  __syncthreads();
+  if (warp == 0) {
+    const float2 t = hqs_reflector(A, 0, p, lane);
+    if (lane == 0) tau_s[0] = t;
+  }
+  __syncthreads();
+  // factorisation: step j applies H_j^H to columns j+1 .. l-1
+  for (int j = 0; j + 1 < l; ++j) {
+    const float2 tau = tau_s[j];
+    float2 v[RPL];
+    hqs_load_v<RPL>(A + int64_t(j) * p, j, p, lane, v);
+    const bool live = tau.x != 0.f || tau.y != 0.f;
+    const float2 f = make_float2(tau.x, -tau.y);
+    int k = j + 1 + warp;
+    if (warp == 0) {   // look-ahead: column j + 1 first, then its reflector
+      float2* c = A + int64_t(k) * p;
+      if (live) hqs_apply<RPL>(v, c, j, p, f, lane);
+      __syncwarp();
+      const float2 t = hqs_reflector(c, k, p, lane);
+      if (lane == 0) tau_s[k] = t;
+      k += HQS_WARPS;
+    }
+    if (live)
+      for (; k < l; k += HQS_WARPS) hqs_apply<RPL>(v, A + int64_t(k) * p, j, p, f, lane);
+    __syncthreads();
+  }
+  // Q = H_0 ... H_{l-1} [I; 0]: step i applies H_i to columns i+1 .. l-1,
+  // whose first (column i + 1) its owner first turns from reflector storage
+  // into H_{i+1} e_{i+1}
+  for (int i = l - 2; i >= 0; --i) {
+    const float2 tau = tau_s[i];
+    float2 v[RPL];
+    hqs_load_v<RPL>(A + int64_t(i) * p, i, p, lane, v);
+    int k = i + 1 + warp;
+    if (warp == 0) {
+      hqs_materialize(A + int64_t(k) * p, k, p, tau_s[k], lane);
+      __syncwarp();
+    }
+    if (tau.x != 0.f || tau.y != 0.f)
+      for (; k < l; k += HQS_WARPS) hqs_apply<RPL>(v, A + int64_t(k) * p, i, p, tau, lane);
+    __syncthreads();
+  }
+  if (warp == 0) hqs_materialize(A, 0, p, tau_s[0], lane);
+  __syncthreads();
+  for (int e = threadIdx.x; e < p * lfull; e += HQS_THREADS) {
+    const float2 q = e < p * l ? A[e] : make_float2(0.f, 0.f);
+    yr[e] = q.x;
+    yi[e] = q.y;
+  }
+}
+
+template <int RPL>
+int hqs_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols, int64_t batch,
+               cudaStream_t st) {
+  const size_t smem = size_t(p) * l * sizeof(float2);
+  TP_SET_SMEM(householder_shared_kernel<RPL>, smem);
+  {
+    KernelScope ks("householder_qr", st);
+    householder_shared_kernel<RPL><<<unsigned(batch), HQS_THREADS, smem, st>>>(yr, yi, sY, p, l,
+                                                                              lcols);
+  }
+  return launch_status("householder_shared_kernel");
+}
+
 constexpr int HQR_BLOCK = 256;
 
 }  // namespace
@@ -605,6 +773,18 @@ int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int
   g.sp = sp;
   g.weak = weak;
   return hqr_dispatch<HQR_WHOLE>(g, p, batch, st);
+}
+
+int householder_shared_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
+                              int64_t batch, cudaStream_t st) {
+  if (p > HQR_BLOCK || l > HQR_MAX_L || l > p) {
+    set_error("householder_shared: needs l <= p <= %d and l <= %d", HQR_BLOCK, HQR_MAX_L);
+    return TP_EUNSUPPORTED;
+  }
+  if (batch <= 0 || l <= 0) return TP_OK;
+  if (p <= 64) return hqs_launch<2>(yr, yi, sY, p, l, lcols, batch, st);
+  if (p <= 128) return hqs_launch<4>(yr, yi, sY, p, l, lcols, batch, st);
+  return hqs_launch<8>(yr, yi, sY, p, l, lcols, batch, st);
 }
 
 // Scratch of householder_tall_launch: per level below the top the R stack

@@ -40,6 +40,11 @@ int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int
                        bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{},
                        int* weak = nullptr);
 
+// The same QR of slices of at most 256 rows with the sums in the order of the
+// shared-memory form (no split planes, no kept phase).
+int householder_shared_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
+                              int64_t batch, cudaStream_t st);
+
 // The same for contiguous slices of more than 256 rows (slice stride rows * l),
 // with `scratch` of householder_tall_scratch() bytes, 256-byte aligned.  A
 // slice that is all zero or not finite sets TP_DEV_BREAKDOWN and is left zero
@@ -48,5 +53,14 @@ size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch);
 int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
                             int64_t batch, void* scratch, int32_t* status, cudaStream_t st,
                             int* weak = nullptr);
+
+// CholeskyQR2 in float64 (cholqr.cu) of contiguous slices of any number of rows
+// >= l, with `scratch` of cholqr_scratch() bytes, 256-byte aligned.  A Gram
+// matrix that is not positive definite even with a shift (an all-zero or not
+// finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.  weak: as
+// above, and set by any slice that needed the shift.
+size_t cholqr_scratch(int64_t l, int64_t batch);
+int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr);
 
 }  // namespace tp

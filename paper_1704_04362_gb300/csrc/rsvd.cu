@@ -8,7 +8,16 @@
 // The test matrix has random-sign entries from Philox stream 2 (see
 // tsvd_randomized in tprod.h).  orth() is a float32 Householder QR
 // (householder.cu): one CTA per slice of at most 256 rows, a tree of them for
-// taller slices.  Every product with X_hat is a plain
+// taller slices.
+//
+// The l x l Gram matrix of the core is formed in float32, so that singular
+// values below about 2^-12 of the largest are resolved as a group only, unless
+// the power iterations have sorted the columns of Q before (q >= 1: spectra
+// i^-2.5 to 1e-7 of their norm).  With q = 0 such trailing values carry
+// errors of 1e-5 of the norm which follow the rounding of all that comes before,
+// so there X_hat and Q are formed with sums in a fixed order
+// (launch_rdft_in_order, householder_shared_launch, cholqr_launch), whatever
+// forms the other paths take.  Every product with X_hat is a plain
 // column-major batched complex GEMM because X_hat^H is formed once.
 #include <cfloat>
 #include <cmath>
@@ -1008,7 +1017,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
   // X_hat and X_hat^H
   DftGather gx{X, n1 * n2, 1, 1, 0, n1 * n2, nullptr, nullptr, nullptr, 0, n3, Xr, Xi,
                n1 * n2, n1 * n2, nullptr, nullptr, 0};
-  if ((rc = launch_rdft(gx, st))) return rc;
+  if ((rc = q == 0 ? launch_rdft_in_order(gx, st) : launch_rdft(gx, st))) return rc;
   if (!tc) {   // X_hat^H for the CUDA-core products (the split forms take planes)
     KernelScope ks("conj_transpose", st);
     conj_transpose_kernel<<<dim3(unsigned((n1 + 31) / 32), unsigned((n2 + 31) / 32), unsigned(h)),
@@ -1084,15 +1093,19 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
   };
   constexpr size_t kSmemCap = 200 * 1024;
   auto orth = [&](float* yr, float* yi, int64_t rows) {
+    planes_ready = false;
     if (householder_applies(rows, l)) {
+      if (q == 0)
+        return householder_shared_launch(yr, yi, rows * l, int(rows), int(l), sketch_per_freq, h,
+                                         st);
       HqrSplit sp{};
       if (tc) sp = HqrSplit{BP[0], BP[1], BP[2], BP[3], split_ld(rows, prec), bf};
       planes_ready = tc;
       return householder_launch(yr, yi, rows * l, int(rows), int(l), sketch_per_freq, false, h, st,
                                 sp);
     }
-    planes_ready = false;
     // the space from Gr on is written by the core only
+    if (q == 0) return cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
     return householder_tall_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
   };
 

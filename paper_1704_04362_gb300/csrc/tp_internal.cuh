@@ -90,6 +90,7 @@ struct DftGather {
   int out_bf16;                // with the split: the four planes hold bf16 (hi, lo) pairs
 };
 int launch_rdft(const DftGather& g, cudaStream_t st);
+int launch_rdft_in_order(const DftGather& g, cudaStream_t st);   // see dft.cu
 
 // Inverse: out[r + rows*t] = (1/n3) sum over the Hermitian-completed spectrum.
 // Input spectrum in{re,im}[k*in_slice + r], k < h.
