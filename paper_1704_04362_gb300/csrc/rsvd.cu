@@ -8,7 +8,7 @@
 // The test matrix has random-sign entries from Philox stream 2 (see
 // tsvd_randomized in tprod.h).  orth() is a float32 Householder QR
 // (householder.cu): one CTA per slice of at most 256 rows, a tree of them for
-// taller slices.
+// taller slices, whose last one is a float64 CholeskyQR2 instead (cholqr.cu).
 //
 // The l x l Gram matrix of the core is formed in float32, so that singular
 // values below about 2^-12 of the largest are resolved as a group only, unless
@@ -1092,7 +1092,8 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
     return gemm_tc(hermitian, N, cr, ci);
   };
   constexpr size_t kSmemCap = 200 * 1024;
-  auto orth = [&](float* yr, float* yi, int64_t rows) {
+  // last: the orthonormalisation that the singular values see
+  auto orth = [&](float* yr, float* yi, int64_t rows, bool last) {
     planes_ready = false;
     if (householder_applies(rows, l)) {
       if (q == 0)
@@ -1105,7 +1106,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
                                 sp);
     }
     // the space from Gr on is written by the core only
-    if (q == 0) return cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
+    if (last) return cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
     return householder_tall_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
   };
 
@@ -1124,12 +1125,12 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
     if ((rc = launch_status("transpose_split_kernel"))) return rc;
   }
   if ((rc = product(false, Or, Oi, l, Yr, Yi))) return rc;     // Y = X_hat Omega
-  if ((rc = orth(Yr, Yi, n1))) return rc;
+  if ((rc = orth(Yr, Yi, n1, q == 0))) return rc;
   for (int it = 0; it < q; ++it) {
     if ((rc = product(true, Yr, Yi, l, Zr, Zi))) return rc;    // Z = X_hat^H Q
-    if ((rc = orth(Zr, Zi, n2))) return rc;
+    if ((rc = orth(Zr, Zi, n2, false))) return rc;
     if ((rc = product(false, Zr, Zi, l, Yr, Yi))) return rc;   // Y = X_hat Z
-    if ((rc = orth(Yr, Yi, n1))) return rc;
+    if ((rc = orth(Yr, Yi, n1, it + 1 == q))) return rc;
   }
   if ((rc = product(true, Yr, Yi, l, Zr, Zi))) return rc;      // B^H = X_hat^H Q
   const int sweeps = (opts && opts->max_sweeps > 0) ? opts->max_sweeps : 30;
