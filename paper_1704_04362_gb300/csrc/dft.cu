@@ -428,7 +428,9 @@ int launch_product(DftArgs& p, int64_t tubes, const char* name, cudaStream_t st)
   const int fit = std::max(1, int(TABLE_BYTES_MAX / (sizeof(float2) * kp * DN)));
   const int groups = (h + DN - 1) / DN;
   p.parts = (groups + fit - 1) / fit;
-  p.ty = (groups + p.parts - 1) / p.parts;
+  // two groups of outputs at least (the second may be past the spectrum), so
+  // that a thread stages 16 samples of a K tile at most
+  p.ty = std::max(2, (groups + p.parts - 1) / p.parts);
   p.N = p.ty * DN;
   p.parts = (h + p.N - 1) / p.N;
   // 16 to 64 lanes along the tubes: small problems and many outputs take few
@@ -441,10 +443,12 @@ int launch_product(DftArgs& p, int64_t tubes, const char* name, cudaStream_t st)
   const size_t smem = kp * p.N * sizeof(float2) + 4 * DK * bm * sizeof(float) +
                       bm * (sizeof(float*) + sizeof(int64_t) + sizeof(float)) +
                       size_t(p.n3) * sizeof(float2);
-  const int np = int((DK * bm + nt - 1) / nt);   // K-tile samples per thread
+  const int np = int((DK * bm + nt - 1) / nt);   // K-tile samples per thread: 32 / ty
   if (np <= 4) return launch_product_np<INV, 4>(p, tubes, smem, name, st);
   if (np <= 8) return launch_product_np<INV, 8>(p, tubes, smem, name, st);
-  return launch_product_np<INV, 16>(p, tubes, smem, name, st);   // ty >= 3: n3 > 16
+  if (np <= 16) return launch_product_np<INV, 16>(p, tubes, smem, name, st);
+  set_error("dft: %d samples a thread", np);
+  return TP_EUNSUPPORTED;
 }
 
 }  // namespace
@@ -468,13 +472,6 @@ int launch_fft_inv(const float* ire, const float* iim, int64_t rows, int64_t in_
 #define TP_FFT_THRESHOLD 16
 #endif
 constexpr int64_t kFftThreshold = TP_FFT_THRESHOLD;
-// Tubes up to 16 and power-of-two ones up to 128 go through the register
-// transforms (rfft_reg.cu); building with -DTP_REG_FFT=0 keeps them on the direct contraction.
-#ifndef TP_REG_FFT
-#define TP_REG_FFT 1
-#endif
-constexpr bool kRegFft = TP_REG_FFT != 0;
-
 int launch_rdft(const DftGather& g, cudaStream_t st) {
   const bool plain = g.gather_dim == 0 && !g.out_transposed && !g.out_re_lo &&
                      (g.cols == 1 || g.col_stride == g.rows) && g.out_ld == g.rows &&
@@ -486,7 +483,7 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
     return TP_EUNSUPPORTED;
   }
   if (g.rows == 0 || g.cols == 0) return TP_OK;
-  if (kRegFft && rfft_reg_supported(g.n3)) return launch_rfft_reg(g, st);
+  if (rfft_reg_supported(g.n3)) return launch_rfft_reg(g, st);
   if (g.n3 > kFftThreshold && fft_supported(g.n3)) return launch_fft_fwd(g, st);
   if (!g.out_transposed) {
     DftArgs p{};
@@ -513,10 +510,11 @@ int launch_rdft(const DftGather& g, cudaStream_t st) {
 }
 
 // The plain forward transform with every frequency's samples summed in order
-// (tubes of 17 to 256 samples that are no power of two up to 128), for callers
+// (tubes of up to 256 samples that are no power of two up to 128), for callers
 // whose results hang on the rounding of its sums; else launch_rdft.
 int launch_rdft_in_order(const DftGather& g, cudaStream_t st) {
-  if (g.n3 <= 16 || g.n3 > 256 || rfft_reg_supported(g.n3)) return launch_rdft(g, st);
+  const bool pow2 = g.n3 <= 128 && (g.n3 & (g.n3 - 1)) == 0;
+  if (g.n3 < 1 || g.n3 > 256 || pow2) return launch_rdft(g, st);
   if (g.rows == 0 || g.cols == 0) return TP_OK;
   DftArgs p{};
   p.g = g;
@@ -531,7 +529,7 @@ int launch_irdft(const float* in_re, const float* in_im, int64_t rows, int64_t i
     return TP_EUNSUPPORTED;
   }
   if (rows == 0) return TP_OK;
-  if (kRegFft && rfft_reg_supported(n3))
+  if (rfft_reg_supported(n3))
     return launch_irfft_reg(in_re, in_im, rows, in_slice, n3, out, st);
   if (n3 > kFftThreshold && fft_supported(n3))
     return launch_fft_inv(in_re, in_im, rows, in_slice, n3, out, st);

@@ -71,3 +71,18 @@ def test_recorded_spectra_decay_past_the_gram_matrix():
 def test_values_are_the_recorded_ones(case):
     got, ref = spectrum(case).ravel().astype(np.float64), recorded()[case].astype(np.float64)
     assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n3", [3, 5, 6, 7, 9, 11, 12, 15])
+def test_short_tubes_match_the_oracle(n3):
+    """Lengths whose product has one or two groups of outputs (a flat spectrum,
+    which every order of the sums resolves; tolerance of the float32 paths)."""
+    from oracle import decomp_ref, philox_ref
+    from paper_1704_04362_gb300 import synth
+    from tests.util import TOL_FP32, rel_fro
+    X = synth.lowrank_np(70, 50, n3, 50, seed=n3, factor="normal")
+    omega = philox_ref.sketch_signs(50, 17, n3 // 2 + 1, n3, 4)
+    ref = decomp_ref.tsvd_randomized_hat(X.astype(np.float64), 17, 0, 0, omega)[1].T
+    got = tp.sketch_spectrum(tp.as_tprod_layout(X), 17, 0, seed=4).cpu().numpy()
+    assert rel_fro(got, ref) < TOL_FP32
