@@ -18,7 +18,8 @@ struct SvtTopArgs {
   const double* mu;
   int* attempt;            // per slice: this iteration tries (Gram needed)
   int* fast;               // per slice, set here: 1 = thresholded here, 0 = takes the Jacobi
-  int* wait;               // per slice: iterations until the next attempt
+  int* wait;               // per slice: iterations until the next attempt, and the
+                           // failed attempts in a row from bit 16 on
   float* edge;             // per slice: smallest kept eigenvalue, 0 = no quadratic filter
   unsigned* above;         // per slice: bit j set = vector j is above the threshold
   int q;
