@@ -220,10 +220,10 @@ int tsvd_randomized(const float* X, int64_t n1, int64_t n2, int64_t n3,
  * slice as P_k A_hat_k with P_k the projector onto range(C_hat_k), whose
  * basis is the left singular vectors of C_hat_k (float64 Jacobi) above
  * MATLAB's pinv cut-off max(n1, c') eps(s_max) or, where up to 96 picked
- * slices (c' <= n1) are clearly of full rank in every frequency, a Householder
- * QR of C_hat_k.
+ * slices (c' <= n1) are clearly of full rank in every frequency, a float64
+ * CholeskyQR2 of C_hat_k.
  *   idx_out / count_out: as tprod_sampled.
- * Reads the pick count, and with the QR its rank check, back to the host
+ * Reads the pick count, and with the CholeskyQR2 its rank check, back to the host
  * (synchronises `stream`).
  * Limits: min(n1, n2) <= 512, n2 <= 4096, n3 <= 512.                        */
 int tcx(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint64_t seed,

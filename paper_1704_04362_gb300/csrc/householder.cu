@@ -241,7 +241,6 @@ struct HqrParams {
   const int* ex_in;        // exponents of this level's source blocks (lfull rows each) or null
   int* flag;               // [slice]: 0, 1 (zero), 2 (not finite)
   int32_t* status;
-  int* weak;               // see householder.cuh
 };
 
 __device__ __forceinline__ void hqr_block(int rows, int nb, int b, int& r0, int& p) {
@@ -411,24 +410,6 @@ __global__ void __launch_bounds__(32 * W, HqrResident<R2, W, SLOTS>::v)
       g.flag[f] = bad;
       if (bad && g.status) atomicOr(g.status, TP_DEV_BREAKDOWN);
     }
-  }
-  if (g.weak && warp == 0) {
-    float lo = INFINITY, hi = 0.f;
-    bool nan = false;
-    for (int j = lane; j < l; j += 32) {
-      const float a = fabsf(beta_s[j]);
-      nan |= isnan(a);
-      lo = fminf(lo, a);
-      hi = fmaxf(hi, a);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    nan = __any_sync(0xffffffffu, nan);
-    const bool sound = !nan && lo > HQR_WEAK * hi && hi > 0x1p-40f && hi < 0x1p40f;
-    if (lane == 0 && !sound) atomicOr(g.weak, 1);
   }
   // Q's column k: H_k e_k = e_k - tau_k v_k, then H_{k-1}, ..., H_0
 #pragma unroll
@@ -755,7 +736,7 @@ constexpr int HQR_BLOCK = 256;
 bool householder_applies(int64_t p, int64_t l) { return p <= HQR_BLOCK && l <= HQR_MAX_L; }
 
 int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
-                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp, int* weak) {
+                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp) {
   if (p > HQR_BLOCK || l > HQR_MAX_L || l > p) {
     set_error("householder: needs l <= p <= %d and l <= %d", HQR_BLOCK, HQR_MAX_L);
     return TP_EUNSUPPORTED;
@@ -771,7 +752,6 @@ int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int
   g.lcols = lcols;
   g.keep_phase = keep_phase ? 1 : 0;
   g.sp = sp;
-  g.weak = weak;
   return hqr_dispatch<HQR_WHOLE>(g, p, batch, st);
 }
 
@@ -801,8 +781,7 @@ size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch) {
 }
 
 int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
-                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st,
-                            int* weak) {
+                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st) {
   constexpr int kMaxLevels = 24;   // each level shrinks the rows by 256 / 96 at least
   if (l < 1 || l > HQR_MAX_L || rows <= HQR_BLOCK || rows > 0x7fffffff) {
     set_error("householder_tall: needs more than %d rows and l <= %d", HQR_BLOCK, HQR_MAX_L);
@@ -828,8 +807,7 @@ int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int
     g.ex_in = ex;
     g.flag = flag;
     g.status = status;
-    g.weak = weak;
-    if (batch * g.nb > 0x7fffffff || (g.nb > 1 && n == kMaxLevels)) {
+      if (batch * g.nb > 0x7fffffff || (g.nb > 1 && n == kMaxLevels)) {
       set_error("householder_tall: too many blocks");
       return TP_EUNSUPPORTED;
     }

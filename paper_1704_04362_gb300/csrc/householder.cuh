@@ -7,12 +7,6 @@ namespace tp {
 
 constexpr int HQR_MAX_L = 96;   // columns of a slice
 
-// weak (device, or null) of the launches below is set to 1 if some slice's
-// diagonal of R leaves the rank in doubt: min |R(j, j)| <= HQR_WEAK max
-// |R(j, j)|, or a maximum outside 2^-40 .. 2^40 (where float32 squares stop
-// being safe) or not finite.  2^-16 is 256 times float32's rounding.
-constexpr float HQR_WEAK = 1.f / 65536.f;
-
 // Split planes (p0 non-null): Q also leaves as the hi/lo planes (bf16 or
 // tf32, dftc::put_split) of the next tensor-core product's B operand,
 // K-major with leading dimension ldk, p <= ldk <= 32 ceil(p / 32) (rows
@@ -37,8 +31,7 @@ bool householder_applies(int64_t p, int64_t l);
 // nearly orthonormal columns Q(:, j) stays close to Y(:, j) instead of
 // possibly flipping its sign.
 int householder_launch(float* yr, float* yi, int64_t sY, int p, int l, const int32_t* lcols,
-                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{},
-                       int* weak = nullptr);
+                       bool keep_phase, int64_t batch, cudaStream_t st, HqrSplit sp = HqrSplit{});
 
 // The same QR of slices of at most 256 rows with the sums in the order of the
 // shared-memory form (no split planes, no kept phase).
@@ -51,16 +44,21 @@ int householder_shared_launch(float* yr, float* yi, int64_t sY, int p, int l, co
 // (not a number).
 size_t householder_tall_scratch(int64_t rows, int64_t l, int64_t batch);
 int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols,
-                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st,
-                            int* weak = nullptr);
+                            int64_t batch, void* scratch, int32_t* status, cudaStream_t st);
 
 // CholeskyQR2 in float64 (cholqr.cu) of contiguous slices of any number of rows
 // >= l, with `scratch` of cholqr_scratch() bytes, 256-byte aligned.  A Gram
 // matrix that is not positive definite even with a shift (an all-zero or not
-// finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.  weak: as
-// above, and set by any slice that needed the shift.
+// finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.
+// settled > 0: the second pass is left out for a slice whose Gram matrix is the
+// identity to that after the first.  weak (device, or null) is set to 1 if some
+// slice's diagonal of R leaves the rank in doubt: a Cholesky breakdown, or min
+// R(j, j) <= CHOLQR_WEAK max R(j, j).  2^-16 is 256 times float32's rounding, and
+// its square is far above float64's.
+constexpr float CHOLQR_WEAK = 1.f / 65536.f;
 size_t cholqr_scratch(int64_t l, int64_t batch);
 int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
-                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr);
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr,
+                  double settled = 0.0);
 
 }  // namespace tp

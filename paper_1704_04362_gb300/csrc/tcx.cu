@@ -9,17 +9,15 @@
 // float32-sweeps + float64-refinement one of svd.cu (float64 accuracy).  The
 // number of picks is read back to the host once (the SVD is sized by it).
 //
-// Where C_hat_k has full column rank, its range is that of any QR's Q, and the
-// SVD is not needed: up to 96 picks (and c' <= n1) the columns are
-// orthonormalised by the Householder QR instead.  Its backward error is of the
-// size of the float32 rounding of C_hat_k itself, so P_k A_hat_k is as accurate
-// as with the SVD of the rounded C_hat_k (measured alike for condition numbers
-// 3e2 .. 4e7).  The diagonal of R tells whether the rank is in doubt
-// (householder.cuh); one slice in doubt sends the call to the SVD, which
-// costs a second read-back and the QR (256 x 512 x 32, 64 picks, one of them a
-// copy: 4.72 -> 4.84 ms a call).
-// The same without the copy: 3.96 -> 0.29 ms a call, half of it the QR's chain
-// of 64 dependent reflectors on 17 SMs.
+// Where C_hat_k has full column rank, its range is that of any orthonormal basis
+// of its columns, and the SVD is not needed: up to 96 picks (and c' <= n1) the
+// basis comes from CholeskyQR in float64 (cholqr.cu), so that P_k is as accurate
+// as with the SVD.  (A float32 Householder QR is quicker, 0.29 ms a call below,
+// but adds its rounding of C_hat_k: 2.4e-7 -> 3.6e-7 to 4.2e-7 -> 5.0e-7 on eight
+// cases.)  R's diagonal tells whether the rank is in doubt (householder.cuh); one
+// slice in doubt sends the call to the SVD, which costs a second read-back and
+// the factorisation.
+// 256 x 512 x 32, 56 to 76 picks: 3.96 (SVD) -> 1.0 to 1.6 ms a call.
 #include <cmath>
 
 #include "householder.cuh"
@@ -204,10 +202,7 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
     if ((r = launch_cgemm(g2, st))) return r;
     return launch_irdft(Zr, Zi, n1 * n2, n1 * n2, n3, Z, st);
   };
-  // the tree's scratch for n1 > 256 lies in the SVD's work matrices
-  const bool tall = !householder_applies(n1, cprime);
-  if (cprime <= n1 && cprime <= HQR_MAX_L && n1 <= 0x7fffffff &&
-      (!tall || householder_tall_scratch(n1, cprime, h) <= 2 * ws_bytes(size_t(P_cap) * m_cap * h, 8))) {
+  if (cprime <= n1 && cprime <= HQR_MAX_L && n1 <= 0x7fffffff && h <= 65535) {
     int* weak = reinterpret_cast<int*>(qsig);
     if (cudaMemsetAsync(weak, 0, sizeof(int), st) != cudaSuccess) {
       set_error("tcx: cudaMemsetAsync failed");
@@ -218,10 +213,9 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
       work_kernel<<<grid_n(n1 * cprime * h), 256, 0, st>>>(Cr, Ci, n1, cprime, n1, n1 * n2, h, false,
                                                            Br, Bi);
     }
-    rc = tall ? householder_tall_launch(Br, Bi, n1, int(cprime), nullptr, h, Gr, nullptr, st, weak)
-              : householder_launch(Br, Bi, n1 * cprime, int(n1), int(cprime), nullptr, false, h, st,
-                                   HqrSplit{}, weak);
-    if (rc) return rc;
+    // scratch in the SVD's G and W; 2^-25: the rounding of Q itself
+    if ((rc = cholqr_launch(Br, Bi, n1, int(cprime), nullptr, h, Gr, nullptr, st, weak, 0x1p-25)))
+      return rc;
     {
       KernelScope ks("tcx_work", st);
       work_kernel<<<grid_n(n1 * cprime * h), 256, 0, st>>>(Br, Bi, n1, cprime, n1, n1 * cprime, h,
