@@ -242,6 +242,7 @@ int tprod_sampled(const float* A, const float* B, float* Z, int64_t n1, int64_t 
           opts ? opts->pipeline_wait_limit : 0};
   if (split && !lean)
     g.split_ws = ws.take<float>(cgemm_split_floats(n1, n4, h, n2, prec));
+  g.kexpect = c;   // c independent draws, or at most c kept slices on average
   if ((rc = launch_cgemm(g, st))) return rc;
   // S7: inverse transform
   return launch_irdft(Zr, Zi, n1 * n4, n1 * n4, n3, Z, st);

@@ -214,6 +214,9 @@ __device__ __forceinline__ int part_begin(int nch, int splits, int sp) {
   return nch / splits * sp + min(sp, nch % splits);
 }
 
+// Parts that hold a chunk (one at least: K = 0 is a part of zeros).
+__device__ __forceinline__ int live_parts(int splits, int nch) { return max(1, min(splits, nch)); }
+
 // Ten warps: two of the four SM sub-partitions hold three of them, and a
 // sub-partition's 16K registers then allow 170 per thread; the epilogue's
 // 128 float32 accumulators fit with 8-column TMEM loads.
@@ -243,7 +246,9 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
   const int tiles_per_f = p.mt * p.nt;
   const int64_t ntiles = int64_t(tiles_per_f) * p.h;
   const int nch = (nkb + KCB - 1) / KCB;   // accumulation chunks per tile
-  const int splits = PARTS ? p.splits : 1;   // work item: tile * splits + part
+  // work item: tile * splits + part; parts past the chunks of a K smaller than
+  // expected would be empty
+  const int splits = PARTS ? live_parts(p.splits, nch) : 1;
   const int64_t nitems = ntiles * splits;
 
   if (threadIdx.x == 0) {
@@ -475,10 +480,13 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(const __grid_constant
   }
 }
 
-// C = the sum of the K parts of every output (planes of n per part, in order).
+// C = the sum of the K parts of every output (planes of n per part, in order;
+// the parts that the product wrote, for a K of `chunk` elements a chunk).
 __global__ void __launch_bounds__(256) cgemm_parts_kernel(const float* __restrict__ part, int64_t n,
                                                           int64_t s_split, int splits,
-                                                          float* __restrict__ out) {
+                                                          const int64_t* __restrict__ dynK,
+                                                          int chunk, float* __restrict__ out) {
+  if (dynK) splits = live_parts(splits, int((*dynK + chunk - 1) / chunk));
   for (int64_t e = int64_t(blockIdx.x) * 256 + threadIdx.x; e < n; e += int64_t(gridDim.x) * 256) {
     float a = part[e];
     for (int sp = 1; sp < splits; ++sp) a += part[e + sp * s_split];
@@ -486,13 +494,20 @@ __global__ void __launch_bounds__(256) cgemm_parts_kernel(const float* __restric
   }
 }
 
+// K elements of an accumulation chunk.
+int64_t cgemm_chunk(int precision) { return int64_t(KCB) * ROWB / (precision == TP_BF16X3 ? 2 : 4); }
+
 // Parts of K for a product with few output tiles: as many as fill the SMs
-// once, at most one per accumulation chunk.  Sized for GB300's 152 SMs
+// once, at most one per accumulation chunk, from three chunks on (the launches
+// that add the parts cost as much as a chunk: sampled products of 100 x 4000 x
+// 100 to 256 x 4000 x 256, whole against cut, us a call: two chunks 46 .. 49
+// against 49 .. 53, four 58 .. 62 against 50 .. 53).  Sized for GB300's 152 SMs
 // wherever it runs, so that a workspace query needs no device.
-int cgemm_splits(int64_t M, int64_t N, int64_t h, int64_t kcap, int precision) {
+int cgemm_splits(int64_t M, int64_t N, int64_t h, int64_t K, int precision) {
   const int64_t tiles = (M + TM - 1) / TM * ((N + TN - 1) / TN) * h;
-  const int64_t chunk = int64_t(KCB) * ROWB / (precision == TP_BF16X3 ? 2 : 4);
-  const int64_t chunks = (kcap + chunk - 1) / chunk;
+  const int64_t chunk = cgemm_chunk(precision);
+  const int64_t chunks = (K + chunk - 1) / chunk;
+  if (chunks < 3) return 1;
   int64_t s = 152 / (tiles < 1 ? 1 : tiles);
   if (s > chunks) s = chunks;
   return s < 2 ? 1 : int(s > 64 ? 64 : s);
@@ -602,9 +617,11 @@ int launch_cgemm_tc(const CGemm& g, cudaStream_t st) {
   p.status = g.status;
   p.mt = int((g.M + TM - 1) / TM);
   p.nt = int((g.N + TN - 1) / TN);
-  // parts of K where the caller gave room for them (and C is contiguous)
+  // parts of K where the caller gave room for them (and C is contiguous); a K
+  // on the device counts as what the caller expects of it, not as its capacity
+  const int64_t K = !g.dynK ? g.K : g.kexpect > 0 ? std::min(g.kexpect, g.kcap) : g.kcap;
   const int splits = g.split_ws && !g.only && g.ldc == g.M && g.sC == g.M * g.N
-                         ? cgemm_splits(g.M, g.N, g.h, g.dynK ? g.kcap : g.K, g.precision)
+                         ? cgemm_splits(g.M, g.N, g.h, K, g.precision)
                          : 1;
   p.splits = splits;
   p.s_split = splits > 1 ? g.M * g.N * g.h : 0;
@@ -631,8 +648,8 @@ int launch_cgemm_tc(const CGemm& g, cudaStream_t st) {
   const unsigned blocks = unsigned(std::min<int64_t>((n + 255) / 256, int64_t(sms) * 8));
   for (int pl = 0; pl < 2; ++pl) {
     KernelScope ks("cgemm_parts", st);
-    cgemm_parts_kernel<<<blocks, 256, 0, st>>>(pl ? p.zi : p.zr, n, p.s_split, splits,
-                                               pl ? g.ci : g.cr);
+    cgemm_parts_kernel<<<blocks, 256, 0, st>>>(pl ? p.zi : p.zr, n, p.s_split, splits, g.dynK,
+                                               int(cgemm_chunk(g.precision)), pl ? g.ci : g.cr);
   }
   return launch_status("cgemm_parts_kernel");
 }

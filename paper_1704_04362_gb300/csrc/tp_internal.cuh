@@ -128,6 +128,8 @@ struct CGemm {
   // tensor-core path: room for the partial sums of a K cut into parts
   // (cgemm_split_floats()), or null: K is not cut
   float* split_ws = nullptr;
+  // with dynK: the K to plan the parts for (0: the capacity)
+  int64_t kexpect = 0;
 };
 // Floats a tensor-core product wants for its K parts (0: it is not cut).
 size_t cgemm_split_floats(int64_t M, int64_t N, int64_t h, int64_t kcap, int precision);
