@@ -658,10 +658,11 @@ __host__ __device__ __forceinline__ int jpc_block_vals(int p, int q) {
   return (n + V - 1) / V * V;
 }
 
+constexpr size_t RING_SMEM_MAX = size_t(200) * 1024;
 template <class T>
 size_t jacobi_ring_smem(int p, int q) {
   const size_t bytes = 4 * size_t(jpc_block_vals<T>(p, q)) * sizeof(T);
-  return bytes <= size_t(200) * 1024 ? bytes : 0;
+  return bytes <= RING_SMEM_MAX ? bytes : 0;
 }
 
 // CTA and slot (0: I, 1: J) of block B in a round.
@@ -1068,6 +1069,45 @@ bool cluster_fits() {
   return v == 1;
 }
 
+// Clusters of a form's kernel that are resident at once with `smem` bytes of
+// shared memory a CTA (0: none can be placed, or the device did not say).
+int resident_clusters(const void* kernel, size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(JPC, 1, 1);
+  cfg.blockDim = dim3(JPC_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;   // the cluster size comes from the kernel's __cluster_dims__
+  int n = 0;
+  if ((smem > 0 && set_smem_attr(kernel, smem, "jacobi_ring_kernel") != TP_OK) ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// Whether `batch` slices take at most num / den times as many rounds of resident
+// clusters in the ring form, with all the shared memory it may ask for, as in
+// the form through L2.  The two counts are asked for once per device.
+bool ring_rounds(int batch, int num, int den) {
+  constexpr int kMaxDev = 64;
+  static std::atomic<unsigned> cache[kMaxDev];   // 0 unknown, else ring << 16 | L2 form | 1 << 31
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+    cudaGetLastError();
+    return false;
+  }
+  unsigned v = cache[dev].load(std::memory_order_relaxed);
+  if (v == 0) {
+    const unsigned ring = unsigned(resident_clusters((const void*)jacobi_ring_kernel<double, 0>, RING_SMEM_MAX));
+    const unsigned l2 = unsigned(resident_clusters((const void*)jacobi_cluster_kernel<float, false>, 0));
+    v = 1u << 31 | (ring & 0x7fff) << 16 | (l2 & 0xffff);
+    cache[dev].store(v, std::memory_order_relaxed);
+  }
+  const int ring = int(v >> 16 & 0x7fff), l2 = int(v & 0xffff);
+  if (ring == 0 || l2 == 0) return false;
+  return (batch + ring - 1) / ring * den <= (batch + l2 - 1) / l2 * num;
+}
+
 // A cluster of CTAs per slice pays when the slices are fewer than the SMs and
 // wide enough to give every CTA of the cluster a block pair of columns.
 bool use_cluster(int q, int batch) {
@@ -1080,13 +1120,19 @@ int jacobi_cluster_launch(T* gr, T* gi, int64_t sG, T* vr, T* vi, int64_t sV, T*
                           int32_t* status, int flags, cudaStream_t st,
                           const int* skip = nullptr) {
   if (batch <= 0 || q <= 0) return TP_OK;
-  // The ring where it is the faster one: float32 pairs that fit the registers
-  // (120 x 100 x 6: 1.91 -> 1.13 ms), or enough columns that a round's rotations
-  // outweigh pushing its columns (256 x 200: float32 5.05 -> 3.95, float64 15.3
-  // and 15.4 ms; 256 x 150 float64 16.9 -> 13.3).  256 x 64 through L2 against the
-  // ring: float32 1.41 / 1.52, float64 1.99 / 2.32 ms.
+  // The ring where it is the faster one: float32 pairs that fit the registers or
+  // enough columns that a round's rotations outweigh pushing its columns, and few
+  // enough slices: it holds an SM per CTA, the form through L2 half of one.
+  // The form through L2 against the ring, ms: float32 13 slices (one round of both) of
+  // 64 x 48 0.565 / 0.360, 128 x 96 1.34 / 0.85, 256 x 96 1.66 / 1.18, 256 x 200
+  // 5.05 / 3.95, 512 x 96 2.16 / 1.50 (float64 128 x 96 2.13 / 1.99); 17 slices (one
+  // and two) 0.62 / 0.67, 1.60 / 1.69, 2.09 / 2.20, 7.71 / 7.33, 3.02 / 3.04; 33 slices (one
+  // and three) 0.62 / 0.96, 1.61 / 2.46, 2.08 / 3.15, 8.5 / 11.2, 2.94 / 4.38; 41 slices
+  // (two and three) 1.16 / 0.99, 2.81 / 2.57, 3.35 / 3.20, 11.55 / 11.46, 4.74 / 4.39
+  // (float64 6.13 / 5.94, 8.40 / 8.56).  13 slices of 256 x 64: 0.94 / 1.5.
   constexpr bool f32 = sizeof(T) == 4;
-  const bool faster = (f32 && std::max(p, q) <= 128) || q >= 96;
+  const bool faster = ((f32 && std::max(p, q) <= 128) || q >= 96) &&
+                      ring_rounds(batch, f32 ? 3 : 1, f32 ? 2 : 1);
   const size_t smem = jacobi_cluster_smem<T>(p, q), ring = faster ? jacobi_ring_smem<T>(p, q) : 0;
   const unsigned grid = unsigned(batch) * JPC;
   {
