@@ -428,9 +428,11 @@ int launch_product(DftArgs& p, int64_t tubes, const char* name, cudaStream_t st)
   const int fit = std::max(1, int(TABLE_BYTES_MAX / (sizeof(float2) * kp * DN)));
   const int groups = (h + DN - 1) / DN;
   p.parts = (groups + fit - 1) / fit;
-  // two groups of outputs at least (the second may be past the spectrum), so
-  // that a thread stages 16 samples of a K tile at most
-  p.ty = std::max(2, (groups + p.parts - 1) / p.parts);
+  // four groups of outputs at least (some may be past the spectrum), so that a
+  // thread stages 8 samples of a K tile at most: n3 = 17, 19, 23 with three groups
+  // and 11 samples, 220000 tubes, forward 28.8, 29.0, 31.7 -> 22.3, 22.7, 24.7 us,
+  // inverse 21.1, 22.3, 22.5 -> 17.5, 17.8, 18.6
+  p.ty = std::max(4, (groups + p.parts - 1) / p.parts);
   p.N = p.ty * DN;
   p.parts = (h + p.N - 1) / p.N;
   // 16 to 64 lanes along the tubes: small problems and many outputs take few
@@ -446,7 +448,6 @@ int launch_product(DftArgs& p, int64_t tubes, const char* name, cudaStream_t st)
   const int np = int((DK * bm + nt - 1) / nt);   // K-tile samples per thread: 32 / ty
   if (np <= 4) return launch_product_np<INV, 4>(p, tubes, smem, name, st);
   if (np <= 8) return launch_product_np<INV, 8>(p, tubes, smem, name, st);
-  if (np <= 16) return launch_product_np<INV, 16>(p, tubes, smem, name, st);
   set_error("dft: %d samples a thread", np);
   return TP_EUNSUPPORTED;
 }
@@ -466,8 +467,7 @@ int launch_fft_inv(const float* ire, const float* iim, int64_t rows, int64_t in_
 // length factors into primes up to 13; building with another value keeps
 // shorter ones on the direct contraction.  218880 tubes, FFT against product,
 // forward / inverse in us: n3 = 80 57 / 53 against 123 / 84; n3 = 225 (odd: a
-// full complex transform) 183 / 247 against 657 / 419; n3 = 45 on 237679 tubes
-// and less 27 / 47 against 45 / 46; level below.
+// full complex transform) 183 / 247 against 657 / 419.
 #ifndef TP_FFT_THRESHOLD
 #define TP_FFT_THRESHOLD 16
 #endif
@@ -531,7 +531,13 @@ int launch_irdft(const float* in_re, const float* in_im, int64_t rows, int64_t i
   if (rows == 0) return TP_OK;
   if (rfft_reg_supported(n3))
     return launch_irfft_reg(in_re, in_im, rows, in_slice, n3, out, st);
-  if (n3 > kFftThreshold && fft_supported(n3))
+  // An odd length is a full complex transform in the FFT, where many tubes leave
+  // the product ahead.  FFT against product, us: n3 = 25, 39, 45 on 32768 tubes 10.4 /
+  // 10.0, 12.5 / 12.4, 12.7 / 12.3, on 49152 11.2 / 9.8, 14.6 / 12.4, 14.5 / 13.7, on
+  // 220000 23.6 / 18.2, 38.9 / 28.8, 41.4 / 32.3; n3 = 49, 63, 75 on 128000 25.6 / 28.1,
+  // 30.8 / 26.5, 39.2 / 39.1, on 220000 43.2 / 44.3, 60.4 / 44.8, 76.1 / 64.6.
+  const bool odd_product = n3 % 2 == 1 && ((n3 < 48 && rows >= 49152) || (n3 < 80 && rows >= 163840));
+  if (n3 > kFftThreshold && fft_supported(n3) && !odd_product)
     return launch_fft_inv(in_re, in_im, rows, in_slice, n3, out, st);
   DftArgs p{};
   p.in_re = in_re;
