@@ -230,11 +230,16 @@ int launch_shape(const CGemm& g, cudaStream_t st) {
 // 56 against 64 us; 64 x 32 x 48, 9 slices: 8.2 against 8.3; but 611 x 389 x
 // 150, 23 slices, ten tiles per SM: 186 against 176).  Larger thread blocks
 // of 8 x 8 outputs were no faster (2819 against 2677 us on the headline shape
-// below).  Both shapes sum in the same order.
+// below).  32 x 32 ones too where C has at most 32 rows or columns, half of a 64
+// x 64 tile or more being work for nothing: 10^6 x 4 x 4, 2 slices 254 -> 145 us, 2000 x 20 x
+// 2000, 9 slices 405 -> 279, 5000 x 10 x 300, 17 slices 274 -> 170.  Both shapes sum
+// in the same order.
 int launch_cgemm_simt(const CGemm& g, cudaStream_t st) {
   if (g.M == 0 || g.N == 0 || g.h == 0) return TP_OK;
   const int64_t K = g.dynK ? g.kcap : g.K;
-  if (K <= 256 && tiles<Wide>(g) < 4 * int64_t(sm_count())) return launch_shape<Small>(g, st);
+  const bool narrow = (g.N <= 32 || g.M <= 32) && g.N <= 32 * int64_t(65535);
+  if (narrow || (K <= 256 && tiles<Wide>(g) < 4 * int64_t(sm_count())))
+    return launch_shape<Small>(g, st);
   return launch_shape<Wide>(g, st);
 }
 
