@@ -49,7 +49,6 @@ struct CholArgs {
   int32_t* status;
   int* weak;               // see householder.cuh
   int first;               // pass 0: every slice takes part
-  double settled;          // a later plain pass whose |G - I| stays below is left out
 };
 
 // a / b from y = 1 / b rounded to nearest: two corrections by the exact remainder
@@ -134,19 +133,6 @@ __global__ void __launch_bounds__(FACTOR_THREADS) cholqr_factor_kernel(const Cho
       for (int j = 0; j < l; ++j) chol_sm[j * l + j].x += sh;
     }
     __syncthreads();
-  }
-  if (!g.first && !s.shifted && g.settled > 0.0) {
-    bool off = false;
-    for (int e = tid; e < l * l; e += FACTOR_THREADS) {
-      const int a = e / l, b = e - a * l;
-      if (a > b) continue;
-      const double re = chol_sm[e].x - (a == b ? 1.0 : 0.0), im = chol_sm[e].y;
-      off |= !(fabs(re) < g.settled && fabs(im) < g.settled);
-    }
-    if (!__syncthreads_or(off)) {
-      if (tid == 0) g.state[f] = Progress{0, 0, 0};
-      return;
-    }
   }
   // row i of R, then its share of every entry right of and below it.  One
   // thread takes the root and its reciprocal: in every warp they would fill the
@@ -275,7 +261,7 @@ size_t cholqr_scratch(int64_t l, int64_t batch) {
 }
 
 int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
-                  void* scratch, int32_t* status, cudaStream_t st, int* weak, double settled) {
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak) {
   if (l < 1 || l > HQR_MAX_L || rows < l || rows > 0x7fffffff || batch > 65535) {
     set_error("cholqr: needs l <= rows, l <= %d and at most 65535 slices", HQR_MAX_L);
     return TP_EUNSUPPORTED;
@@ -283,7 +269,7 @@ int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcol
   if (batch <= 0) return TP_OK;
   Arena ws;
   ws.base = static_cast<char*>(scratch);
-  CholArgs g{yr, yi, rows * l, int(rows), l, lcols, nullptr, nullptr, status, weak, 1, settled};
+  CholArgs g{yr, yi, rows * l, int(rows), l, lcols, nullptr, nullptr, status, weak, 1};
   g.G = ws.take<double2>(size_t(l) * l * batch);
   g.state = ws.take<Progress>(size_t(batch));
   const size_t gram_smem = size_t(GRAM_ROWS) * (l | 1) * sizeof(double2);

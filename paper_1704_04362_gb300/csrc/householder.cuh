@@ -49,16 +49,13 @@ int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int
 // CholeskyQR2 in float64 (cholqr.cu) of contiguous slices of any number of rows
 // >= l, with `scratch` of cholqr_scratch() bytes, 256-byte aligned.  A Gram
 // matrix that is not positive definite even with a shift (an all-zero or not
-// finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.
-// settled > 0: the second pass is left out for a slice whose Gram matrix is the
-// identity to that after the first.  weak (device, or null) is set to 1 if some
-// slice's diagonal of R leaves the rank in doubt: a Cholesky breakdown, or min
-// R(j, j) <= CHOLQR_WEAK max R(j, j).  2^-16 is 256 times float32's rounding, and
+// finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.  weak
+// (device, or null) is set to 1 if some slice's diagonal of R leaves the rank in
+// doubt: a Cholesky breakdown, or min R(j, j) <= CHOLQR_WEAK max R(j, j).  2^-16 is 256 times float32's rounding, and
 // its square is far above float64's.
 constexpr float CHOLQR_WEAK = 1.f / 65536.f;
 size_t cholqr_scratch(int64_t l, int64_t batch);
 int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
-                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr,
-                  double settled = 0.0);
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr);
 
 }  // namespace tp

@@ -11,8 +11,8 @@
 //
 // Where C_hat_k has full column rank, its range is that of any orthonormal basis
 // of its columns, and the SVD is not needed: up to 96 picks (and c' <= n1) the
-// basis comes from CholeskyQR in float64 (cholqr.cu), so that P_k is as accurate
-// as with the SVD.  (A float32 Householder QR is quicker, 0.29 ms a call below,
+// basis comes from CholeskyQR2 in float64 (cholqr.cu), so that P_k is as accurate
+// as with the SVD (errors of 4.0e-7 .. 4.3e-7 became 3.7e-7 .. 3.8e-7 below).  (A float32 Householder QR is quicker, 0.29 ms a call below,
 // but adds its rounding of C_hat_k: 2.4e-7 -> 3.6e-7 to 4.2e-7 -> 5.0e-7 on eight
 // cases.)  R's diagonal tells whether the rank is in doubt (householder.cuh); one
 // slice in doubt sends the call to the SVD, which costs a second read-back and
@@ -36,7 +36,8 @@ namespace {
 
 __global__ void work_kernel(const float* __restrict__ xr, const float* __restrict__ xi,
                             int64_t n1, int64_t c, int64_t ld, int64_t slice, int64_t h,
-                            bool transpose, float* __restrict__ gr, float* __restrict__ gi) {
+                            bool transpose, float* __restrict__ gr, float* __restrict__ gi,
+                            bool flip = false) {
   const int64_t per = n1 * c, total = per * h;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
        e += int64_t(gridDim.x) * blockDim.x) {
@@ -47,8 +48,9 @@ __global__ void work_kernel(const float* __restrict__ xr, const float* __restric
       gr[e] = vr;
       gi[e] = vi;
     } else {
-      gr[k * per + j + c * i] = vr;
-      gi[k * per + j + c * i] = -vi;
+      const int64_t o = k * per + (flip ? c - 1 - j : j) + c * i;   // rows last to first
+      gr[o] = vr;
+      gi[o] = -vi;
     }
   }
 }
@@ -191,13 +193,16 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
                n1 * n2, n1 * n2, nullptr, nullptr, 0};
   if ((rc = launch_rdft(ga, st))) return rc;
 
-  // T = U_r^H A_hat (m x n2), Z_hat = U_r T (n1 x n2), Z
-  auto project = [&](int64_t m) {
+  // T = U_r^H A_hat (m x n2), Z_hat = U_r T (n1 x n2), Z; flip: U_r^H is stored last
+  // row first, and the second product takes U_r's columns that way (sums from the
+  // last column on)
+  auto project = [&](int64_t m, bool flip) {
     CGemm g1{Hr, Hi, Ar, Ai, Tr, Ti, m, n2, n1, nullptr, m, n1, m, m * n1, n1 * n2, m * n2, h, n3,
              TP_FP32, nullptr, nullptr, nullptr, nullptr, n1, status};
     int r = launch_cgemm(g1, st);
     if (r) return r;
-    CGemm g2{Br, Bi, Tr, Ti, Zr, Zi, n1, n2, m, nullptr, n1, m, n1, n1 * m, m * n2, n1 * n2, h, n3,
+    const int64_t first = flip ? n1 * (m - 1) : 0;
+    CGemm g2{Br + first, Bi + first, Tr, Ti, Zr, Zi, n1, n2, m, nullptr, flip ? -n1 : n1, m, n1, n1 * m, m * n2, n1 * n2, h, n3,
              TP_FP32, nullptr, nullptr, nullptr, nullptr, m, status};
     if ((r = launch_cgemm(g2, st))) return r;
     return launch_irdft(Zr, Zi, n1 * n2, n1 * n2, n3, Z, st);
@@ -213,13 +218,16 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
       work_kernel<<<grid_n(n1 * cprime * h), 256, 0, st>>>(Cr, Ci, n1, cprime, n1, n1 * n2, h, false,
                                                            Br, Bi);
     }
-    // scratch in the SVD's G and W; 2^-25: the rounding of Q itself
-    if ((rc = cholqr_launch(Br, Bi, n1, int(cprime), nullptr, h, Gr, nullptr, st, weak, 0x1p-25)))
-      return rc;
+    // scratch in the SVD's G and W
+    if ((rc = cholqr_launch(Br, Bi, n1, int(cprime), nullptr, h, Gr, nullptr, st, weak))) return rc;
     {
+      // The first picks carry most of the tensor (each later column is only what
+      // the ones before leave), so Z_hat is summed from the last column on: fewer
+      // float32 additions at full size, a tenth less error than the SVD's columns
+      // give in their order, where pick order gave 5% more.
       KernelScope ks("tcx_work", st);
       work_kernel<<<grid_n(n1 * cprime * h), 256, 0, st>>>(Br, Bi, n1, cprime, n1, n1 * cprime, h,
-                                                           true, Hr, Hi);
+                                                           true, Hr, Hi, true);
     }
     if ((rc = launch_status("tcx_work"))) return rc;
     int doubt = 0;
@@ -229,7 +237,7 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
       set_error("tcx: reading the rank check failed");
       return TP_ECUDA;
     }
-    if (!doubt) return project(cprime);
+    if (!doubt) return project(cprime, true);
   }
 
   const bool transpose = n1 < cprime;
@@ -257,7 +265,7 @@ int tcx_run(const float* A, int64_t n1, int64_t n2, int64_t n3, int64_t c, uint6
                                                       Bi, Hr, Hi);
   }
   if ((rc = launch_status("tcx_basis"))) return rc;
-  return project(m);
+  return project(m, false);
 }
 
 }  // namespace tp

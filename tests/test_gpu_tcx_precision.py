@@ -2,9 +2,9 @@
 it.  A duplicate of one picked slice sends the call to the SVD and leaves the
 span as it is, so the two errors against the float64 projection are of the same
 result: float32 rounding of the tensor, of the basis and of the products in both.
-Allowed: a tenth more on the mean over the cases (each error is a root mean
-square over thousands of entries, so that means of the same roundings differ by
-less)."""
+The mean over the cases may not be larger than the SVD's (each error is a root
+mean square over thousands of entries; the sums that start with the small
+columns make it a tenth smaller)."""
 import numpy as np
 import pytest
 
@@ -35,4 +35,4 @@ def test_error_is_the_svd_forms():
         A = np.asfortranarray(A.astype(np.float32))
         plain.append(error(A, list(range(c))))
         svd.append(error(A, list(range(c)) + [n2 - 1]))
-    assert np.mean(plain) <= 1.1 * np.mean(svd), (plain, svd)
+    assert np.mean(plain) <= np.mean(svd), (plain, svd)
