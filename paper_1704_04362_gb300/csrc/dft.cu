@@ -45,7 +45,7 @@ __device__ __forceinline__ void build_twiddles(float2* tw, int n3) {
 // K x 4 TY table of the transform matrix stays in shared memory while the
 // block walks its tubes; the tubes come in K tiles of 8, folded on the way from
 // registers to shared memory, the next tile's samples loaded before the
-// current one is used.  The whole half spectrum of a tube up to n3 = 256 is
+// current one is used.  The whole half spectrum of a tube of up to 239 samples is
 // produced by one block, so each sample is read once (longer tubes take the
 // outputs in as many parts as their table needs shared memory).
 // Bound by the float32 pipe for n3 above about 60, below by the tubes' traffic.
@@ -55,7 +55,7 @@ __device__ __forceinline__ void build_twiddles(float2* tw, int n3) {
 constexpr int DK = 8;                        // K tile
 constexpr int DN = 4, DM = 4;                // outputs and tubes per thread
 constexpr int TABLE_BYTES_MAX = 120 * 1024;
-constexpr int DT_MAX = 544;                  // threads: 16 x 33 at n3 = 256
+constexpr int DT_MAX = 480;                  // threads: 16 x 30 groups, n3 = 232 .. 239
 
 struct DftArgs {
   DftGather g;                // forward

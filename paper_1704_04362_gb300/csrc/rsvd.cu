@@ -2,7 +2,8 @@
 // finder with power iterations of Halko, Martinsson and Tropp (2011):
 //   Y = X_hat Omega;  Q = orth(Y)
 //   q times: Z = orth(X_hat^H Q), Q = orth(X_hat Z)
-//   B^H = X_hat^H Q  (n2 x l);  B^H = V_B diag(s) W^H (one-sided Jacobi, float64)
+//   B^H = X_hat^H Q  (n2 x l);  B^H = V_B diag(s) W^H (W from the l x l Gram matrix's
+//   Householder tridiagonalisation and implicit QL in float32, s = ||B^H w||)
 //   U_f = Q W[:, :k],  V_f = V_B[:, :k],  S_f = diag(s[:k])
 // followed by the inverse DFT of U, S, V (Theorem 2.6's form, tubal rank k).
 // The test matrix has random-sign entries from Philox stream 2 (see

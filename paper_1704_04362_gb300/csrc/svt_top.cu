@@ -24,9 +24,10 @@
 // One CTA per slice: Q and Y in shared memory, G read from L2 (packed
 // two-lane FMAs, a row x 8 columns a thread), the Cholesky in place in G
 // by panels of 32 columns.
-// Bound by the loads of the products (a row's 8 columns need 3 shared-memory
-// and 2 global loads per 16 packed FMAs) and by the certificate's panels, one
-// after the other, half the time each.
+// Bound by one block's share of an SM: of a slice's 1.35 M cycles the products
+// with G take a third (bound by their loads, 3 from shared and 2 from global
+// memory per 16 packed FMAs of a row's 8 columns), the certificate's panels a
+// fifth, the 32 x 32 Jacobi a sixth, small products, sums and factors the rest.
 // 41 slices of 144 x 256 (the 144 x 256 x 80 completion), one iteration: 3.5 ms
 // by the warm-started Jacobi and its GEMMs -> 0.53 ms here and 0.14 ms of GEMMs.
 // From 48 columns on (below, the Jacobi's slices are small and many fit an
