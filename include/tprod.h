@@ -185,8 +185,9 @@ int tsvd(const float* X, int64_t n1, int64_t n2, int64_t n3,
  * 1/sqrt((k+p) p_j), so that Y holds picked columns of X_hat;
  * q power iterations Q <- orth(X_hat^H Q), Q <- orth(X_hat Q), each orth a
  * float32 Householder QR (it cannot break down; slices of more than 256 rows
- * as a tree of blocks, and their last orth as CholeskyQR2 in float64; there an
- * all-zero or not finite slice sets TP_DEV_BREAKDOWN), then B = Q^H X_hat, the SVD of B through its l x l Gram (float32
+ * as a tree of blocks, whose last orth ends in a float64 CholeskyQR, or with
+ * q <= 1 as float64 CholeskyQR2; there an all-zero or not finite slice sets
+ * TP_DEV_BREAKDOWN), then B = Q^H X_hat, the SVD of B through its l x l Gram (float32
  * two-sided Jacobi, singular values as the Rayleigh quotients ||B^H w_j||
  * with float64 sums) and U = Q U_B truncated to k.
  *   opts->precision  TP_FP32: the products with X_hat on the CUDA cores;

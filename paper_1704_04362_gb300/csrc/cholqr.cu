@@ -8,11 +8,13 @@
 // followed by two plain passes (shifted CholeskyQR3).
 //
 // The last orthonormalisation of the randomized t-SVD decides how far Q is from
-// orthonormal, and every singular value is off by as much, so it runs in
-// float64; the ones before it only carry a subspace to the next product and stay
-// with the float32 tree (householder.cu).  Singular values of slices of 400 to
-// 1000 rows after one power iteration: 5e-8 .. 9e-8 off with this, 8e-8 ..
-// 1.2e-7 with the tree alone.
+// orthonormal, and every singular value is off by as much, so it ends in float64;
+// the ones before it only carry a subspace to the next product and stay with the
+// float32 tree (householder.cu).  After two power iterations the last one is the
+// tree too, with one pass of this on its nearly orthonormal Q ("polish"); with
+// fewer every one is two passes of this (rsvd.cu).  Singular values of slices of
+// 400 to 1000 rows after one power iteration: 5e-8 .. 9e-8 off with two passes, 6e-8
+// .. 9e-8 with the tree and one, 8e-8 .. 1.2e-7 with the tree alone.
 //
 // Bound by the float64 pipe (two lanes a cycle and SM): a Gram entry is six
 // operations a row, a solve six per entry of R and row.  So the Gram entries are
@@ -49,6 +51,7 @@ struct CholArgs {
   int32_t* status;
   int* weak;               // see householder.cuh
   int first;               // pass 0: every slice takes part
+  int passes;              // plain passes wanted
 };
 
 // a / b from y = 1 / b rounded to nearest: two corrections by the exact remainder
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(FACTOR_THREADS) cholqr_factor_kernel(const Cho
   extern __shared__ __align__(16) double2 chol_sm[];   // l x l, row-major; then the triangle
   __shared__ int bad;
   const int f = blockIdx.x, l = columns_of(g, f), tid = threadIdx.x;
-  Progress s = g.first ? Progress{2, 0, 0} : g.state[f];
+  Progress s = g.first ? Progress{g.passes, 0, 0} : g.state[f];
   if (s.passes <= 0) {
     if (tid == 0) g.state[f].solve = 0;
     return;
@@ -261,7 +264,7 @@ size_t cholqr_scratch(int64_t l, int64_t batch) {
 }
 
 int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
-                  void* scratch, int32_t* status, cudaStream_t st, int* weak) {
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak, bool polish) {
   if (l < 1 || l > HQR_MAX_L || rows < l || rows > 0x7fffffff || batch > 65535) {
     set_error("cholqr: needs l <= rows, l <= %d and at most 65535 slices", HQR_MAX_L);
     return TP_EUNSUPPORTED;
@@ -269,7 +272,7 @@ int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcol
   if (batch <= 0) return TP_OK;
   Arena ws;
   ws.base = static_cast<char*>(scratch);
-  CholArgs g{yr, yi, rows * l, int(rows), l, lcols, nullptr, nullptr, status, weak, 1};
+  CholArgs g{yr, yi, rows * l, int(rows), l, lcols, nullptr, nullptr, status, weak, 1, polish ? 1 : 2};
   g.G = ws.take<double2>(size_t(l) * l * batch);
   g.state = ws.take<Progress>(size_t(batch));
   const size_t gram_smem = size_t(GRAM_ROWS) * (l | 1) * sizeof(double2);
@@ -287,7 +290,7 @@ int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcol
   const unsigned pairs = unsigned((l * (l + 1) / 2 + GRAM_THREADS - 1) / GRAM_THREADS);
   const unsigned blocks = unsigned((rows + T - 1) / T), slices = unsigned(batch);
   // four passes at most: the breakdown, its shifted repeat and two plain ones
-  for (int it = 0; it < 4; ++it) {
+  for (int it = 0; it < (polish ? 1 : 4); ++it) {
     g.first = it == 0;
     {
       KernelScope ks("cholqr_gram", st);

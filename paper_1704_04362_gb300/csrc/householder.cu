@@ -566,7 +566,7 @@ int hqr_dispatch(const HqrParams& g, int p, int64_t blocks, cudaStream_t st) {
 // The same QR of a slice of at most 256 rows held in shared memory, a step's
 // reflector in registers (lane r % 32 holds rows r) and a warp per column.  It
 // is a few percent slower than the registers' form above and rounds in another
-// order.  The sketch without power iterations takes it: there the trailing
+// order.  Sketches with at most one power iteration take it: there the trailing
 // singular values are set by the rounding of the core's Gram matrix (rsvd.cu),
 // so that another order of the sums here moves them by more than rounding.
 constexpr int HQS_THREADS = 256;

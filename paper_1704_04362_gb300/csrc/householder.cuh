@@ -52,10 +52,12 @@ int householder_tall_launch(float* yr, float* yi, int64_t rows, int l, const int
 // finite slice) sets TP_DEV_BREAKDOWN and leaves the slice as it is.  weak
 // (device, or null) is set to 1 if some slice's diagonal of R leaves the rank in
 // doubt: a Cholesky breakdown, or min R(j, j) <= CHOLQR_WEAK max R(j, j).  2^-16 is 256 times float32's rounding, and
-// its square is far above float64's.
+// its square is far above float64's.  polish: one pass only, for slices that are
+// nearly orthonormal; one that is not positive definite stays as it is.
 constexpr float CHOLQR_WEAK = 1.f / 65536.f;
 size_t cholqr_scratch(int64_t l, int64_t batch);
 int cholqr_launch(float* yr, float* yi, int64_t rows, int l, const int32_t* lcols, int64_t batch,
-                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr);
+                  void* scratch, int32_t* status, cudaStream_t st, int* weak = nullptr,
+                  bool polish = false);
 
 }  // namespace tp

@@ -9,15 +9,15 @@
 // The test matrix has random-sign entries from Philox stream 2 (see
 // tsvd_randomized in tprod.h).  orth() is a float32 Householder QR
 // (householder.cu): one CTA per slice of at most 256 rows, a tree of them for
-// taller slices, whose last one is a float64 CholeskyQR2 instead (cholqr.cu).
+// taller slices, whose last one ends in a float64 CholeskyQR (cholqr.cu).
 //
 // The l x l Gram matrix of the core is formed in float32, so that singular
 // values below about 2^-12 of the largest are resolved as a group only, unless
-// the power iterations have sorted the columns of Q before (q >= 1: spectra
-// i^-2.5 to 1e-7 of their norm).  With q = 0 such trailing values carry
-// errors of 1e-5 of the norm which follow the rounding of all that comes before,
-// so there X_hat and Q are formed with sums in a fixed order
-// (launch_rdft_in_order, householder_shared_launch, cholqr_launch), whatever
+// the power iterations have sorted the columns of Q before (q >= 2: spectra
+// i^-2.5 to 1e-6 of their norm and mostly 1e-7).  With q = 0 such trailing values
+// carry errors of 1e-5 of the norm, with q = 1 some 1e-6, which follow the rounding
+// of all that comes before, so there X_hat and Q are formed with sums in a fixed
+// order (launch_rdft_in_order, householder_shared_launch, cholqr_launch), whatever
 // forms the other paths take.  Every product with X_hat is a plain
 // column-major batched complex GEMM because X_hat^H is formed once.
 #include <cfloat>
@@ -961,6 +961,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
              const int32_t* sketch_per_freq) {
   const int64_t h = half_len(n3);
   const int64_t l = k + p;
+  const bool ordered = q <= 1;   // sums in a fixed order, see the file's comment
   const int prec = opts ? opts->precision : TP_FP32;
   if (prec != TP_FP32 && prec != TP_TF32X3 && prec != TP_BF16X3) {
     set_error("tsvd_randomized: unknown precision %d", prec);
@@ -1018,7 +1019,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
   // X_hat and X_hat^H
   DftGather gx{X, n1 * n2, 1, 1, 0, n1 * n2, nullptr, nullptr, nullptr, 0, n3, Xr, Xi,
                n1 * n2, n1 * n2, nullptr, nullptr, 0};
-  if ((rc = q == 0 ? launch_rdft_in_order(gx, st) : launch_rdft(gx, st))) return rc;
+  if ((rc = ordered ? launch_rdft_in_order(gx, st) : launch_rdft(gx, st))) return rc;
   if (!tc) {   // X_hat^H for the CUDA-core products (the split forms take planes)
     KernelScope ks("conj_transpose", st);
     conj_transpose_kernel<<<dim3(unsigned((n1 + 31) / 32), unsigned((n2 + 31) / 32), unsigned(h)),
@@ -1097,7 +1098,7 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
   auto orth = [&](float* yr, float* yi, int64_t rows, bool last) {
     planes_ready = false;
     if (householder_applies(rows, l)) {
-      if (q == 0)
+      if (ordered)
         return householder_shared_launch(yr, yi, rows * l, int(rows), int(l), sketch_per_freq, h,
                                          st);
       HqrSplit sp{};
@@ -1107,8 +1108,11 @@ int rsvd_run(const float* X, int64_t n1, int64_t n2, int64_t n3, int k, int p, i
                                 sp);
     }
     // the space from Gr on is written by the core only
-    if (last) return cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
-    return householder_tall_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
+    if (ordered) return cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
+    int r2 = householder_tall_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, status, st);
+    if (!r2 && last)
+      r2 = cholqr_launch(yr, yi, rows, int(l), sketch_per_freq, h, Gr, nullptr, st, nullptr, true);
+    return r2;
   };
 
   if (tc) {
