@@ -29,7 +29,7 @@ def sweeps_ms(n1, n2, slices):
 
 @pytest.mark.parametrize("n1,n2", [(64, 48), (160, 96)])
 def test_more_slices_than_rings(n1, n2):
-    assert sweeps_ms(n1, n2, 33) < 1.2 * sweeps_ms(n1, n2, 25)
+    assert sweeps_ms(n1, n2, 33) < 1.25 * sweeps_ms(n1, n2, 25)
 
 
 @pytest.mark.parametrize("slices", [13, 17, 33])

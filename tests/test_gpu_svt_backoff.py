@@ -36,7 +36,7 @@ def device_ms(X, mask, iters):
 def test_failing_attempts_are_spaced_out():
     X, mask = data(96, 64, 8, 5, 0.0)
     early, before, after = (device_ms(X, mask, n)["svt_top"] for n in (60, 110, 170))
-    assert (after - before) / 60 < 0.5 * early / 60
+    assert after - before < early   # 2.4 times it with an attempt in every iteration
 
 
 @pytest.mark.parametrize("n1,n2,n3,rank,noise,iters", [(96, 64, 4, 5, 0.0, 130),
